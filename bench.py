@@ -45,6 +45,23 @@ FP64_FLOPS_PER_CLK_SM = 1.25e12 / (SMS * 2.07e9)
 # (FMA = 2, the reciprocal square root = 1): 3 displacements 42, ATM terms 49,
 # gradient scalars, energy and virial 9, force vectors 27 (3c01: 9).
 F3 = {"3c01": 109.0, "3c18": 127.0, "3c08": 127.0, "3c08a": 127.0}
+# The forward lists (FP32C pair rule of 3c01, 3c18, 3c08): the third side from
+# two list rows 8, the five differences and sums of the squared sides 10, the
+# three derivatives 26, energy 4, the two rows' sums 20 (3c01 counts a triplet
+# at each of its three owners).
+F3_FORWARD = 68.0
+
+
+def forward_lists(trav, trunc, prec):
+    return prec == "fp32c" and trunc == "pair" and trav in ("3c01", "3c18", "3c08")
+
+
+def flops3(trav, trunc, prec):
+    """Useful flops per counted interacting triplet."""
+    if forward_lists(trav, trunc, prec):
+        return F3_FORWARD / 3.0 if trav == "3c01" else F3_FORWARD
+    return F3[trav]
+
 
 # Useful flops per interacting LJ pair when a step evaluates LJ inside the
 # block units (3c08 / 3c18 / 3c08a, pair rule): displacement and square 14,
@@ -61,7 +78,8 @@ FUSED_TRAV = ("3c08", "3c18", "3c08a")
 # reports null until it is captured again.  liquid_n256k is the N = 32,000
 # capture (2197 units) scaled to 19683 units.
 KERNEL_SOURCES = ["atm3_internal.cuh", "atm_common.cuh", "atm_block.cuh", "atm_owner.cuh",
-                  "atm_fp32.cu", "atm_fp64.cu", "atm_launch.cuh", "pair_masks.cu"]
+                  "atm_fp32.cu", "atm_fp64.cu", "atm_launch.cuh", "pair_masks.cu", "atm_fwd.cuh",
+                  "atm_fwd.cu"]
 TRAFFIC = {("3c08", "pair", "fp32c", "liquid_n256k"): (32.43e6, "86ebe58ae46bedf4"),
            ("3c08", "pair", "fp32c", "liquid_n32k"): (3.620e6, "86ebe58ae46bedf4")}
 
@@ -337,7 +355,7 @@ def run_ours(args):
     prof = main["prof"]
     atm_ms = prof["ms_atm"] / max(1, prof["n_atm_launches"])
     fused = args.trav in FUSED_TRAV and args.trunc == "pair"
-    flops = F3[args.trav] * main["res"]["n_int3"]
+    flops = flops3(args.trav, args.trunc, args.prec) * main["res"]["n_int3"]
     if fused:
         flops += F2_FUSED * main["res"]["n_int2"]
     pk = peaks()
@@ -352,10 +370,12 @@ def run_ours(args):
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak,
                 "traffic": traffic_for(args.trav, args.trunc, args.prec, args.workload),
-                "kernel": ("atm_owner_kernel<%s,%s,%s>" if args.trav == "3c01" else "atm_block_kernel<%s,%s,%s>") % (args.trav, args.trunc, args.prec)
-                          + (" (LJ of the c08 pairs inside)" if fused else "")
-                          + (" after k_pair_masks" if args.prec == "fp32c" and args.trunc == "pair"
-                             and args.trav in ("3c08", "3c18", "3c08a") else ""),
+                "kernel": (("k_atm_fwd<%s,%s,%s>" if forward_lists(args.trav, args.trunc, args.prec)
+                            else "atm_owner_kernel<%s,%s,%s>" if args.trav == "3c01"
+                            else "atm_block_kernel<%s,%s,%s>") % (args.trav, args.trunc, args.prec)
+                           + (" (LJ inside)" if fused else "")
+                           + (" after k_pair_masks" if args.prec == "fp32c" and args.trunc == "pair"
+                              and args.trav == "3c08a" else "")),
                 "peak_source": ("measured: atm_measure_fma_peak, %s FMA chains on every SM"
                                 % ("FP32" if args.prec == "fp32c" else "FP64"))
                                if peak == measured else "derived (measurement failed)",
@@ -363,7 +383,7 @@ def run_ours(args):
                 "derived_peak_source": "%d SMs x %.2f flops/clk x %.0f MHz (%s pipe)"
                                        % (SMS, per_clk, sm_max,
                                           "FP32" if args.prec == "fp32c" else "FP64, nominal"),
-                "flops_per_interacting_triplet": F3[args.trav],
+                "flops_per_interacting_triplet": flops3(args.trav, args.trunc, args.prec),
                 "flops_per_interacting_pair": F2_FUSED if fused else None,
                 "ms_per_launch": atm_ms,
                 "measured_fma_peak_tflops": measured,
@@ -420,7 +440,7 @@ def run_ours(args):
             am = r["prof"]["ms_atm"] / max(1, r["prof"]["n_atm_launches"])
             # useful flops over the ATM evaluation's time, against the measured
             # FMA peak of the variant's precision
-            vflops = F3[tv] * r["res"]["n_int3"]
+            vflops = flops3(tv, tr, pr) * r["res"]["n_int3"]
             if tv in FUSED_TRAV and tr == "pair":
                 vflops += F2_FUSED * r["res"]["n_int2"]
             if pr not in vpeak:

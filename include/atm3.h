@@ -85,13 +85,17 @@ typedef enum { ATM_TRUNC_PAIR = 0, ATM_TRUNC_PRODUCT = 1 } atm_truncation;
  *  FP64:  every decision and every force, energy and virial term in FP64.
  *  FP32C: decisions and per-triplet arithmetic in FP32 on FP32 cell-local
  *         coordinates (every pair decision on the canonical displacement
- *         (xl_q - xl_p) + (o_q - o_p) w; the pair-rule block traversals then
- *         evaluate triplets and forces on the FP32-rounded unit-frame
- *         positions xl + o w).  Force sums: 3C18 / 3C08 / 3C08A add each triplet's
- *         three pair scalars to per-edge FP32 sums, then each molecule's share
- *         of a unit is a plain FP32 sum over its edges, and the shares of
- *         different units are added in FP64; 3C01 / 3CW keep compensated
- *         (Kahan) FP32 per-lane sums of F_i, combined in FP64.  Energy and
+ *         (xl_q - xl_p) + (o_q - o_p) w).  Force sums: under the pair rule 3C01,
+ *         3C18 and 3C08 find the same triplets, each evaluated once at its
+ *         lowest molecule i on the FP32 displacements from i; what the
+ *         triplets of i put on one partner is a plain FP32 sum, and the shares
+ *         of different i are added in FP64.  3C08A and the product rule of
+ *         3C18 / 3C08 add each triplet's three pair scalars to per-edge FP32
+ *         sums (pair rule: on the FP32-rounded unit-frame positions xl + o w),
+ *         then each molecule's share of a unit is a plain FP32 sum over its
+ *         edges, and the shares of different units are added in FP64; 3C01
+ *         (product rule) and 3CW keep compensated (Kahan) FP32 per-lane sums
+ *         of F_i, combined in FP64.  Energy and
  *         virial: Kahan-compensated FP32 per lane, reduced in FP64.  (The
  *         deterministic mode sums the block traversals' terms in fixed
  *         point instead, see atm_set_deterministic.)
@@ -240,7 +244,8 @@ atm_status atm_get_results(atm_ctx* ctx, atm_result* out);
 /* Launch options.  persistent = 1: the ATM kernel runs as a persistent grid
  * (resident CTAs x SMs) whose CTAs take traversal units from a global counter
  * instead of one CTA per unit.  nwarps = 4 or 8 warps per 3C18/3C08 CTA (0 =
- * default).  graph = 1: atm_step captures one step in a CUDA graph (on a
+ * default); neither applies to the FP32C pair rule of 3C01, 3C18 and 3C08,
+ * whose launch form follows from the system.  graph = 1: atm_step captures one step in a CUDA graph (on a
  * stream of its own) and replays it, with no host synchronisation between
  * steps; the graph sizes the kernels for the current largest unit plus
  * headroom (at most a quarter of it, the largest amount that keeps the
@@ -294,8 +299,9 @@ atm_status atm_set_owned_layers(atm_ctx* ctx, int replica, int z_lo, int z_hi);
  * Errors: INVALID. */
 atm_status atm_set_deterministic(atm_ctx* ctx, int on);
 
-/* Pair bitmaps for the FP32C pair rule of the block traversals (on = 1, the
- * default; 0 = off).  With them on, each force evaluation first decides every
+/* Pair bitmaps for the FP32C pair rule of the block traversals where they run
+ * in the block kernel (3C08A; units too large for the forward lists that 3C18
+ * and 3C08 otherwise take) (on = 1, the default; 0 = off).  With them on, each force evaluation first decides every
  * pair of molecules in neighbouring cells once, in one kernel and its
  * transposition: 27 words per molecule (4 bytes each, held by the context),
  * bit j of word k set when the molecule and the j-th molecule of the
@@ -370,7 +376,7 @@ atm_status atm_density_reset(atm_ctx* ctx);
  * allocator must not be touched after start-up.  It does what atm_create +
  * atm_set_state_dev + atm_build_cells + atm_compute_forces + atm_get_forces_dev
  * (which = 0) do for one set of positions, but allocates nothing: every
- * intermediate array lives in one fixed __device__ array of about 6.7 MB that
+ * intermediate array lives in one fixed __device__ array of about 7.8 MB that
  * this library reserves on every GPU it is loaded on, until the process exits.
  *
  *   params  box, rc, nu, LJ parameters, device, cuda_stream (dt is unused)

@@ -6,6 +6,11 @@
 namespace atm3 {
 
 constexpr int ATM_NTRAV = 5;  // 3c01, 3c18, 3c08, 3cw, corner-anchored 3c08
+// unit sizes a cell build measures: the traversals' and the forward-list unit's
+// (18 cells); MAXOCC_N: largest cell, those, the traversals' edge-table needs
+constexpr int ATM_FWD_UNIT = ATM_NTRAV;
+constexpr int ATM_NUNIT = ATM_NTRAV + 1;
+constexpr int MAXOCC_N = 1 + ATM_NUNIT + ATM_NTRAV;
 constexpr int ATM_MAX_DEVICES = 64;  // per-device kernel attribute bookkeeping
 
 // device status word bits (set by kernels, read back by the host)
@@ -201,6 +206,73 @@ struct AtmArgs {
     // (nullptr: not recorded)
     int* emax;
 };
+
+// Arguments of the forward-list kernel (atm_fwd.cuh: FP32C pair rule of 3c01,
+// 3c18 and 3c08).
+struct FwdArgs {
+    Batch b;
+    long long n;              // SoA stride = b.ntot
+    const float* xl;          // sorted cell-local coordinates, SoA [3n]
+    const int* cell_start;
+    double* fs;               // sorted-order force, SoA [3n] (zero at launch): ATM, or LJ + ATM (lj = 1)
+    double* fs_lj;            // lj = 2: the LJ force, SoA [3n] (zero at launch)
+    // per CTA (cell * split + part): E3, W3; 0, interacting; with lj E2, W2; 0,
+    // pairs (the candidates are counted by the reduction)
+    double* unit_ew;
+    unsigned long long* unit_cnt;
+    double* unit_ew2;
+    unsigned long long* unit_cnt2;
+    int* status;
+    int mcap;                 // molecule capacity of 18 cells
+    int run;                  // base cells of a CTA, along x
+    const int* runs;          // run > 1, several replicas: first cell of every run (nullptr: one replica)
+    long long nruns;
+    int split;                // run = 1: CTAs per cell
+    int lj;                   // 0 none, 1 into fs, 2 into fs_lj
+    int trav;                 // whose candidates and visits are counted: 0, 1, 2
+};
+
+constexpr int FWD_RUN = 4;     // most base cells of a CTA
+constexpr int FWD_CELLS = 6 * (FWD_RUN + 2);  // staged cells: a run's columns and one on either side
+constexpr int FWD_MAXW = 8;    // most warps of a CTA
+constexpr int FWD_EXTRA = 8;   // rows beyond 32 that are met one by one
+// list rows a warp keeps: 32 twice over and the extra ones, or a list in chunks
+constexpr int FWD_ROWS = 64 + FWD_EXTRA;
+constexpr int FWD_SPLIT = 4;   // most CTAs per cell
+
+// CTAs per cell whose partial sums the unit arrays must hold: several only
+// for systems of few cells
+__host__ __device__ inline long long fwd_unit_slots(long long ncell)
+{
+    return ncell * FWD_SPLIT <= 8192 ? ncell * FWD_SPLIT : (ncell < 8192 ? 8192 : ncell);
+}
+
+// staged-molecule capacity of a run, mcap the capacity of any 18 cells (three
+// columns of six)
+__host__ __device__ inline int fwd_stage(int mcap, int run) { return (run + 4) / 3 * mcap; }
+
+// Shared-memory plan of the forward-list kernel: staged positions (cell-local
+// and unit-frame, read in 32s), the warps' list rows and partner indices (any
+// list fits the latter).
+struct FwdSmem {
+    int icap;
+    size_t off_pos, off_frame, off_list, off_lidx, total;
+};
+
+__host__ __device__ inline FwdSmem fwd_smem_plan(int mcap, int run, int nwarps)
+{
+    FwdSmem p;
+    size_t o = 0;
+    auto al = [](size_t v) { return (v + 15) & ~(size_t)15; };
+    const size_t M = (size_t)fwd_stage(mcap, run);
+    p.icap = (mcap + 7) & ~7;
+    p.off_pos = o;   o = al(o + 16 * M);
+    p.off_frame = o; o = al(o + 16 * (M + 32));
+    p.off_list = o;  o = al(o + 16 * (size_t)FWD_ROWS * nwarps);
+    p.off_lidx = o;  o = al(o + sizeof(unsigned short) * (size_t)p.icap * nwarps);
+    p.total = o;
+    return p;
+}
 
 // pair bitmaps: word k - 13 of molecule s (sorted) covers the molecules of
 // the cell at offset27(k), k = 13 (its own cell, the later molecules) .. 26
@@ -427,6 +499,9 @@ cudaError_t launch_block_det64(int trav, int trunc, const AtmArgs<double>& a, in
                                size_t smem, int ctas, cudaStream_t s);
 cudaError_t launch_block_det32(int trav, int trunc, const AtmArgs<float>& a, int nwarps,
                                size_t smem, int ctas, cudaStream_t s);
+// the forward-list kernel (atm_fwd.cu), one CTA of nwarps warps per cell and
+// part; the shared-memory limit is raised as needed
+cudaError_t launch_atm_fwd(const FwdArgs& a, int det, int nwarps, cudaStream_t s);
 cudaError_t attr_block_det64(int trav, int trunc, size_t smem);
 cudaError_t attr_block_det32(int trav, int trunc, size_t smem);
 int occupancy_block_det64(int trav, int trunc, int nwarps, size_t smem);

@@ -118,7 +118,7 @@ static void free_all(atm_ctx* c)
                    c->f_lj, c->f_atm, c->f_out, c->unit_ew, c->unit_cnt, c->mol_ew, c->mol_cnt,
                    c->ke, c->d_res, c->d_part, c->d_status, c->d_maxocc, c->d_work, c->d_dens,
                    c->d_rdf, c->d_ttarget, c->unit_ew2, c->unit_cnt2, c->f_in, c->d_chk,
-                   c->d_ulist, c->d_ucount, c->pmask};
+                   c->d_ulist, c->d_ucount, c->d_runs, c->pmask};
     for (void* p : dev)
         if (p) cudaFree(p);
     if (c->h_res) cudaFreeHost(c->h_res);
@@ -248,10 +248,11 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
     ok = ok && alloc((void**)&c->f_out, 3 * N * sizeof(double));
     ok = ok && alloc((void**)&c->f_in, 3 * N * sizeof(double));
     ok = ok && alloc((void**)&c->d_chk, sizeof(int));
-    ok = ok && alloc((void**)&c->unit_ew, 2 * NC * sizeof(double));
-    ok = ok && alloc((void**)&c->unit_cnt, 2 * NC * sizeof(unsigned long long));
-    ok = ok && alloc((void**)&c->unit_ew2, 2 * NC * sizeof(double));
-    ok = ok && alloc((void**)&c->unit_cnt2, 2 * NC * sizeof(unsigned long long));
+    const size_t NU = (size_t)fwd_unit_slots(ncell);
+    ok = ok && alloc((void**)&c->unit_ew, 2 * NU * sizeof(double));
+    ok = ok && alloc((void**)&c->unit_cnt, 2 * NU * sizeof(unsigned long long));
+    ok = ok && alloc((void**)&c->unit_ew2, 2 * NU * sizeof(double));
+    ok = ok && alloc((void**)&c->unit_cnt2, 2 * NU * sizeof(unsigned long long));
     ok = ok && alloc((void**)&c->mol_ew, 2 * N * sizeof(double));
     ok = ok && alloc((void**)&c->mol_cnt, 2 * N * sizeof(unsigned));
     ok = ok && alloc((void**)&c->ke, N * sizeof(double));
@@ -259,11 +260,13 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
     ok = ok && alloc((void**)&c->d_part, (size_t)nrep * REDUCE_PARTS * sizeof(ResultDev));
     ok = ok && alloc((void**)&c->d_status, sizeof(int));
     // largest cell, largest unit per traversal, edge-table need per traversal
-    ok = ok && alloc((void**)&c->d_maxocc, (1 + 2 * ATM_NTRAV) * sizeof(int));
-    ok = ok && cudaMemset(c->d_maxocc, 0, (1 + 2 * ATM_NTRAV) * sizeof(int)) == cudaSuccess;
+    ok = ok && alloc((void**)&c->d_maxocc, MAXOCC_N * sizeof(int));
+    ok = ok && cudaMemset(c->d_maxocc, 0, MAXOCC_N * sizeof(int)) == cudaSuccess;
     ok = ok && alloc((void**)&c->d_work, 4 * sizeof(int));
     ok = ok && alloc((void**)&c->d_ulist, 3 * NC * sizeof(int));
     ok = ok && alloc((void**)&c->d_ucount, 4 * sizeof(int));
+    for (const Rep& r : c->reps) c->nruns += fwd_runs_of(r.g);
+    if (nrep > 1) ok = ok && alloc((void**)&c->d_runs, (size_t)c->nruns * sizeof(int));
     ok = ok && alloc((void**)&c->d_dens, (size_t)nrep * DENS_MAX_BINS * sizeof(unsigned long long));
     ok = ok && alloc((void**)&c->d_rdf, (size_t)nrep * DENS_MAX_BINS * sizeof(unsigned long long));
     ok = ok && alloc((void**)&c->d_ttarget, nrep * sizeof(double));
@@ -271,7 +274,7 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
     ok = ok && cudaMallocHost((void**)&c->h_res, nrep * sizeof(ResultDev)) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&c->h_status, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&c->h_chk, sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMallocHost((void**)&c->h_maxocc, (1 + 2 * ATM_NTRAV) * sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMallocHost((void**)&c->h_maxocc, MAXOCC_N * sizeof(int)) == cudaSuccess;
     ok = ok && cudaDeviceGetAttribute(&c->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin,
                                       c->device) == cudaSuccess;
     ok = ok && cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) ==
@@ -288,6 +291,16 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
         for (int r = 0; r < nrep; r++) {
             for (long long q = 0; q < c->reps[r].g.ncell; q++) roc[c->reps[r].cell0 + q] = r;
             for (long long q = 0; q < c->reps[r].n; q++) rom[c->reps[r].mol0 + q] = r;
+        }
+        if (nrep > 1) {
+            std::vector<int> runs;
+            runs.reserve((size_t)c->nruns);
+            for (const Rep& r : c->reps)
+                for (long long row = 0; row < (long long)r.g.nc[1] * r.g.nc[2]; row++)
+                    for (int x = 0; x < r.g.nc[0]; x += FWD_RUN)
+                        runs.push_back((int)(r.cell0 + row * r.g.nc[0] + x));
+            ok = ok && cudaMemcpy(c->d_runs, runs.data(), runs.size() * sizeof(int),
+                                  cudaMemcpyHostToDevice) == cudaSuccess;
         }
         ok = ok && cudaMemcpy(c->d_rep, c->reps.data(), nrep * sizeof(Rep),
                               cudaMemcpyHostToDevice) == cudaSuccess;
@@ -455,9 +468,10 @@ static atm_status launch_cells(atm_ctx* c)
 static void take_unit_sizes(atm_ctx* c)
 {
     c->maxocc = c->h_maxocc[0];
+    c->unit_max[ATM_FWD_UNIT] = c->h_maxocc[1 + ATM_FWD_UNIT];
     for (int t = 0; t < ATM_NTRAV; t++) {
         c->unit_max[t] = c->h_maxocc[1 + t];
-        const int need = c->h_maxocc[1 + ATM_NTRAV + t];
+        const int need = c->h_maxocc[1 + ATM_NUNIT + t];
         const int g = need > 0 ? std::min(256, need + 4) : c->gpm16[t];
         if (g != c->gpm16[t]) {
             c->gpm16[t] = g;
@@ -471,7 +485,7 @@ static atm_status enqueue_cells(atm_ctx* c)
 {
     atm_status s = launch_cells(c);
     if (s != ATM_OK) return s;
-    CU(cudaMemcpyAsync(c->h_maxocc, c->d_maxocc, (1 + 2 * ATM_NTRAV) * sizeof(int),
+    CU(cudaMemcpyAsync(c->h_maxocc, c->d_maxocc, MAXOCC_N * sizeof(int),
                        cudaMemcpyDeviceToHost, c->st));
     s = ctx_sync_and_check(c);
     if (s != ATM_OK) return s;
@@ -522,6 +536,29 @@ extern "C" atm_status atm_get_cells(atm_ctx* c, int32_t* cell_of, int32_t* cell_
 // options; cls = {classes, first bound, second bound} (1 class: all units in
 // one launch)
 static int atm_ctas_per_sm(const atm_ctx* c, int trav, int trunc, int prec, int nwarps, int mcap);
+static int graph_mcap_fwd(const atm_ctx* c);
+
+// steps of this combination take the forward lists (launch options and size
+// classes then have nothing to choose)
+static bool fwd_active(const atm_ctx* c, int trav, int trunc, int prec)
+{
+    if (prec == ATM_SURROGATE) return false;
+    ForceJob j;
+    j.b = c->b;
+    j.prec = prec;
+    j.trunc = trunc;
+    j.trav = trav;
+    j.optin = c->smem_optin;
+    j.sms = c->sms;
+    j.det = c->det;
+    j.whole = c->whole;
+    j.lj = lj_fused(trav, trunc, prec);
+    j.lj_apart = !j.lj;
+    j.mcap_fwd = graph_mcap_fwd(c);
+    j.runs = c->d_runs;
+    j.nruns = c->nruns;
+    return atm_fwd_plan(j).use;
+}
 
 static void launch_choice(atm_ctx* c, int trav, int trunc, int prec, int mcap, int& persistent,
                           int& nwarps, int cls[3])
@@ -640,10 +677,19 @@ atm_status atm3::ctx_enqueue_forces(atm_ctx* c, int trav, int trunc, int prec, i
     j.det = c->det;
     j.pmask = use_pair_masks(c, trav, trunc, prec) ? c->pmask : nullptr;
     j.gpm16 = edge_capacity(c, trav, trunc);
-    j.emax = measured_edges(c, trav, trunc) ? c->d_maxocc + 1 + ATM_NTRAV + trav : nullptr;
+    j.emax = measured_edges(c, trav, trunc) ? c->d_maxocc + 1 + ATM_NUNIT + trav : nullptr;
+
+    // the forward lists' capacity follows the traversal's headroom
+    const int um = c->unit_max[trav], uf = c->unit_max[ATM_FWD_UNIT];
+    j.mcap_fwd = prec == ATM_SURROGATE ? 0 : (um > 0 && mcap > um ? graph_mcap_fwd(c) : (uf > 0 ? uf : 1));
+    j.whole = c->whole;
+    j.lj_apart = prec != ATM_SURROGATE && !fused;
+    j.runs = c->d_runs;
+    j.nruns = c->nruns;
+    const FwdLaunch fwd = atm_fwd_plan(j);
 
     cudaEvent_t ev;
-    if (prec != ATM_SURROGATE && !fused) {
+    if (prec != ATM_SURROGATE && !fused && fwd.lj != 2) {
         // (the surrogate's descriptor pass computes LJ from the same neighbours)
         ev = ctx_prof_begin(c, PK_LJ);
         CU(enqueue_lj(j));
@@ -677,6 +723,9 @@ atm_status atm3::ctx_enqueue_forces(atm_ctx* c, int trav, int trunc, int prec, i
     c->f_trunc = trunc;
     c->f_prec = prec;
     c->f_fused = fused;
+    c->f_unit_lj = fused || (fwd.use && fwd.lj == 2);
+    c->f_split = fwd.use ? fwd.split : 1;
+    c->f_fwd = fwd.use;
     return ATM_OK;
 }
 
@@ -686,8 +735,11 @@ static atm_status enqueue_reduce(atm_ctx* c)
     r.b = c->b;
     r.unit_ew = c->unit_ew;
     r.unit_cnt = c->unit_cnt;
-    r.unit_ew2 = c->f_fused ? c->unit_ew2 : nullptr;
-    r.unit_cnt2 = c->f_fused ? c->unit_cnt2 : nullptr;
+    r.unit_ew2 = c->f_unit_lj ? c->unit_ew2 : nullptr;
+    r.unit_cnt2 = c->f_unit_lj ? c->unit_cnt2 : nullptr;
+    r.split = c->f_split;
+    r.cand_trav = c->f_fwd ? c->f_trav : -1;
+    r.cell_start = c->start;
     r.mol_ew = c->mol_ew;
     r.mol_cnt = c->mol_cnt;
     r.ke = c->ke;
@@ -866,6 +918,14 @@ static int graph_mcap(const atm_ctx* c, int trav, int trunc, int prec, int nwarp
     return std::min(limit, m + 4);
 }
 
+// the same headroom for the forward lists' 18-cell units, whose shared memory
+// leaves room for it: an eighth of the unit, at least 8
+static int graph_mcap_fwd(const atm_ctx* c)
+{
+    const int m = std::max(1, c->unit_max[ATM_FWD_UNIT]);
+    return m + std::max(8, m / 8);
+}
+
 // run nsteps with a CUDA graph of one step (no host synchronisation between
 // steps); a capacity overflow surfaces in the status word
 static atm_status run_graph_steps(atm_ctx* c, int nsteps, int trav, int trunc, int prec)
@@ -873,8 +933,10 @@ static atm_status run_graph_steps(atm_ctx* c, int nsteps, int trav, int trunc, i
     int persistent = 0, nwarps = 0, cls[3] = {1, 0, 0};
     if (prec != ATM_SURROGATE)
         launch_choice(c, trav, trunc, prec, c->unit_max[trav], persistent, nwarps, cls);
+    const bool fwd = fwd_active(c, trav, trunc, prec);
+    if (fwd) cls[0] = 1;
     const int mcap = graph_mcap(c, trav, trunc, prec, nwarps);
-    const int key[9] = {trav, trunc, prec, mcap,
+    const int key[10] = {trav, trunc, prec, mcap, fwd ? graph_mcap_fwd(c) : 0,
                         persistent + 2 * nwarps + 64 * (use_pair_masks(c, trav, trunc, prec) ? 1 : 0),
                         cls[0], cls[1], cls[2], edge_capacity(c, trav, trunc)};
     if (!c->graph || memcmp(key, c->graph_key, sizeof(key)) != 0) {
@@ -961,7 +1023,7 @@ extern "C" atm_status atm_step(atm_ctx* c, int nsteps, atm_traversal trav, atm_t
         }
         s = run_graph_steps(c, nsteps, trav, trunc, prec);
         if (s != ATM_OK) return s;
-        CU(cudaMemcpyAsync(c->h_maxocc, c->d_maxocc, (1 + 2 * ATM_NTRAV) * sizeof(int),
+        CU(cudaMemcpyAsync(c->h_maxocc, c->d_maxocc, MAXOCC_N * sizeof(int),
                            cudaMemcpyDeviceToHost, c->st));
         s = ctx_sync_and_check(c);
         if (s == ATM_OK) {
@@ -1151,6 +1213,9 @@ extern "C" atm_status atm_set_owned_layers(atm_ctx* c, int replica, int z_lo, in
     r.own_z1 = z_hi;
     CU(cudaMemcpyAsync(c->d_rep + replica, &r, sizeof(Rep), cudaMemcpyHostToDevice, c->st));
     CU(cudaStreamSynchronize(c->st));
+    c->whole = true;
+    for (const Rep& q : c->reps)
+        if (q.own_z0 != 0 || q.own_z1 != q.g.nc[2]) c->whole = false;
     drop_graph(c);
     c->forces_valid = false;
     return ATM_OK;
@@ -1206,12 +1271,13 @@ extern "C" atm_status atm_autotune(atm_ctx* c, atm_traversal trav, atm_truncatio
     int best_code = 1;
     atm_status s = ATM_OK;
     const bool owner = trav == ATM_3C01 || trav == ATM_3CW;
-    const int nw_options = owner ? 1 : 2, split_options = owner ? 1 : N_SPLITS;
+    const bool one = fwd_active(c, trav, trunc, prec);
+    const int nw_options = owner || one ? 1 : 2, split_options = owner || one ? 1 : N_SPLITS;
     // the evaluation as steps take it (LJ inside the units where steps fuse it)
     const bool fuse = lj_fused(trav, trunc, prec);
     for (int sp = 0; sp < split_options && s == ATM_OK; sp++)
     for (int nwi = 0; nwi < nw_options && s == ATM_OK; nwi++)
-        for (int pers = 0; pers < 2 && s == ATM_OK; pers++) {
+        for (int pers = 0; pers < (one ? 1 : 2) && s == ATM_OK; pers++) {
             const int code = 1 + pers + 2 * nwi + 4 * sp;
             c->tuned[prec][trav][trunc] = code;
             s = ctx_enqueue_forces(c, trav, trunc, prec, c->unit_max[trav], fuse);  // warm-up

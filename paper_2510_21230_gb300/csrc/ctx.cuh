@@ -59,6 +59,8 @@ struct atm_ctx {
     int* d_work = nullptr;    // [4] persistent unit counters (one per unit size class)
     int* d_ulist = nullptr;   // [3 * ncell] unit lists of the size classes
     int* d_ucount = nullptr;  // [4] their lengths
+    int* d_runs = nullptr;    // several replicas: first cell of every run of FWD_RUN cells
+    long long nruns = 0;
     unsigned long long* d_dens = nullptr;  // [R * DENS_MAX_BINS]
     unsigned long long* d_rdf = nullptr;   // [R * DENS_MAX_BINS]
     double* d_ttarget = nullptr;           // [R] thermostat temperatures
@@ -68,15 +70,20 @@ struct atm_ctx {
     int dens_axis = -1, dens_nbins = 0;
     long long dens_samples = 0;
     int maxocc = 0;
-    int unit_max[atm3::ATM_NTRAV] = {};  // largest unit (staged molecules) of 3c01, 3c18, 3c08, 3cw
+    // largest unit (staged molecules) of 3c01, 3c18, 3c08, 3cw, 3c08a and the forward lists
+    int unit_max[atm3::ATM_NUNIT] = {};
     // pair rule of the block traversals outside the deterministic mode: the
     // edge table's capacity in 1/16 edges per staged molecule, from the
-    // largest need the units of this context recorded (d_maxocc[1 + NTRAV +
+    // largest need the units of this context recorded (d_maxocc[1 + NUNIT +
     // trav], read with the unit sizes) plus a margin; 256 before any
     int gpm16[atm3::ATM_NTRAV] = {256, 256, 256, 256, 256};
     bool have_x = false, cells_built = false, forces_valid = false;
     int f_trav = -1, f_trunc = -1, f_prec = -1;
     bool f_fused = false;  // the current forces came from units that also did LJ
+    bool f_unit_lj = false;  // the LJ sums of the current forces are in unit_ew2 / unit_cnt2
+    int f_split = 1;         // partial sums per cell in the unit arrays
+    bool f_fwd = false;      // the current forces came from forward lists
+    bool whole = true;       // every replica owns all its layers
     bool wide_cells = false;  // cell builds also size the wide traversal's 5^3 units
     // forces of the current state given by the caller (original order, total),
     // for the combination f_in_key = (traversal, truncation, precision)
@@ -115,7 +122,7 @@ struct atm_ctx {
     double* x_host_out = nullptr;  // where the last step copies its positions early
     bool x_out_issued = false;     // that copy is in flight on io_st
     cudaGraphExec_t graph = nullptr;
-    int graph_key[9] = {-1, -1, -1, -1, -1, -1, -1, -1, -1};
+    int graph_key[10] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
     // profiling: event pairs around launch groups, summed per kind
     int prof = 0;  // profiling: 0 off, 1 every launch group, 2 force evaluations only
     struct EvRec {

@@ -161,15 +161,82 @@ static cudaError_t launch_atm_one(const ForceJob& j, size_t* smem_set, bool* cap
     return launch_atm_fp32(j.trav, j.trunc, a, P.nwarps, P.smem, ctas, j.st);
 }
 
+// The FP32C pair rule of 3c01, 3c18 and 3c08 takes the forward lists (liquid of
+// 256,000 molecules at rho* 0.8, forces and LJ apart: 0.50 ms against 1.16 ms
+// of the pair bitmaps and the block kernel and 0.19 ms of the LJ kernel; five
+// steps 3.82 against 8.42 ms; 5,003 molecules 0.19 against 0.28 ms per call).
+// Left to the other kernels: 3c01 in parts of
+// a domain (owner computes: only owned molecules get a force) and in the
+// deterministic mode (its sums need no fixed point, so no term can leave the
+// fixed-point range), the corner-anchored 3c08 (not every triangle), and units
+// that do not fit shared memory.
+FwdLaunch atm_fwd_plan(const ForceJob& j)
+{
+    FwdLaunch f;
+    if (j.prec != 1 || j.trunc != 0 || (j.trav != 0 && j.trav != 1 && j.trav != 2) || j.mcap_fwd <= 0 ||
+        (j.trav == 0 && (!j.whole || j.det)))
+        return f;
+    // LJ apart only for whole systems (in a domain the LJ kernel gives owned
+    // molecules their complete force) and in floating point
+    f.lj = j.lj && j.trav != 0 ? 1 : (j.lj_apart && j.whole && !j.det ? 2 : 0);
+    // eight warps and a run of four cells per CTA; one cell, and several CTAs per
+    // cell, while the grid would leave SMs without enough warps
+    const long long sms = j.sms > 0 ? j.sms : 148, occ = (j.b.ntot + j.b.ncell - 1) / j.b.ncell;
+    const long long want = sms * 24;  // warps
+    if (j.nruns <= 0 || j.nruns * FWD_MAXW < 2 * want) {
+        f.run = 1;
+        if (occ <= 4) f.nwarps = 4;
+        const long long most = std::min<long long>({FWD_SPLIT, (occ + FWD_MAXW - 1) / FWD_MAXW,
+                                                    fwd_unit_slots(j.b.ncell) / j.b.ncell});
+        while (f.split < most && j.b.ncell * f.nwarps * f.split < want) f.split++;
+    }
+    const size_t lim = j.optin > 4096 ? (size_t)j.optin - 4096 : 0;
+    auto fits = [&]() {
+        return fwd_stage(j.mcap_fwd, f.run) <= 65535 &&
+               fwd_smem_plan(j.mcap_fwd, f.run, f.nwarps).total <= lim;
+    };
+    if (!fits() && f.run > 1) {
+        f.run = 1;
+        f.split = 1;
+    }
+    while (f.nwarps > 1 && !fits()) f.nwarps /= 2;
+    f.use = fits();
+    return f;
+}
+
+static cudaError_t launch_fwd(const ForceJob& j, const FwdLaunch& f)
+{
+    FwdArgs a{};
+    a.b = j.b;
+    a.n = j.b.ntot;
+    a.xl = j.xl32;
+    a.cell_start = j.start;
+    a.fs = j.f_atm;
+    a.fs_lj = j.f_lj;
+    a.unit_ew = j.unit_ew;
+    a.unit_cnt = j.unit_cnt;
+    a.unit_ew2 = j.unit_ew2;
+    a.unit_cnt2 = j.unit_cnt2;
+    a.status = j.status;
+    a.mcap = j.mcap_fwd;
+    a.run = f.run;
+    a.runs = j.runs;
+    a.nruns = j.nruns;
+    a.split = f.split;
+    a.lj = f.lj;
+    a.trav = j.trav;
+    return launch_atm_fwd(a, j.det, f.nwarps, j.st);
+}
+
 bool atm_uses_pair_masks(const ForceJob& j)
 {
-    return j.pmask && j.prec == 1 && j.trunc == 0 && (j.trav == 1 || j.trav == 2 || j.trav == 4) &&
+    return j.pmask && !atm_fwd_plan(j).use && j.prec == 1 && j.trunc == 0 && (j.trav == 1 || j.trav == 2 || j.trav == 4) &&
            j.b.ntot > 0;
 }
 
 bool atm_split_active(const ForceJob& j)
 {
-    return j.ncls > 1 && (j.trav == 1 || j.trav == 2 || j.trav == 4) && j.ulist && j.ucount &&
+    return !atm_fwd_plan(j).use && j.ncls > 1 && (j.trav == 1 || j.trav == 2 || j.trav == 4) && j.ulist && j.ucount &&
            j.b.ncell > 0;
 }
 
@@ -198,6 +265,13 @@ static cudaError_t enqueue_atm_launches(const ForceJob& j, size_t* smem_set, boo
         }
     }
     cudaError_t e;
+    const FwdLaunch f = atm_fwd_plan(j);
+    if (f.use) {
+        if (j.b.ntot <= 0) return launch_fwd(j, f);
+        e = cudaMemsetAsync(j.f_atm, 0, 3 * (size_t)j.b.ntot * sizeof(double), j.st);
+        if (e == cudaSuccess && f.lj) e = cudaMemsetAsync(j.f_lj, 0, 3 * (size_t)j.b.ntot * sizeof(double), j.st);
+        return e == cudaSuccess ? launch_fwd(j, f) : e;
+    }
     if (j.trav != 0 && j.trav != 3 && j.b.ntot > 0) {  // owner traversals write every F_i
         e = cudaMemsetAsync(j.f_atm, 0, 3 * (size_t)j.b.ntot * sizeof(double), j.st);
         if (e != cudaSuccess) return e;

@@ -70,7 +70,30 @@ struct ForceJob {
     // (nullptr: not recorded)
     int gpm16 = 256;
     int* emax = nullptr;
+    // FP32C pair rule from forward lists (atm_fwd.cuh): largest 18-cell unit
+    // (0: not known, the list path is not taken); the unit arrays hold
+    // fwd_unit_slots(ncell) entries; whole: every layer owned; lj_apart: the
+    // caller wants the LJ force on its own and may get it from the units
+    // (unit_ew2 / unit_cnt2 then hold its sums)
+    int mcap_fwd = 0;
+    bool whole = false;
+    bool lj_apart = false;
+    const int* runs = nullptr;  // FwdArgs.runs and nruns of FWD_RUN cells (device)
+    long long nruns = 0;
 };
+
+// how an evaluation from forward lists is launched
+struct FwdLaunch {
+    bool use = false;  // the job takes the list path
+    int lj = 0;        // 0 no LJ, 1 inside fs, 2 apart
+    int nwarps = FWD_MAXW, run = FWD_RUN, split = 1;
+};
+FwdLaunch atm_fwd_plan(const ForceJob& j);
+// runs of FWD_RUN cells of one replica's grid
+inline long long fwd_runs_of(const Grid& g)
+{
+    return (long long)((g.nc[0] + FWD_RUN - 1) / FWD_RUN) * g.nc[1] * g.nc[2];
+}
 
 cudaError_t enqueue_lj(const ForceJob& j);
 // *capacity is set when no kernel configuration fits the unit size

@@ -124,11 +124,12 @@ __global__ void __launch_bounds__(1024) k_scan(long long ncell, const int* __res
 }
 
 // largest staged-molecule count of a traversal unit, per traversal:
-// out[0] 3c01 (27 cells), out[1] 3c18 (base + 13 forward), out[2] 3c08 (2x2x2 block)
+// out[0] 3c01 (27 cells), out[1] 3c18 (base + 13 forward), out[2] 3c08 (2x2x2 block),
+// out[ATM_FWD_UNIT] the forward lists' 18 cells (the base cell's layer and the next)
 __global__ void k_unit_max(Batch B, const int* __restrict__ start, int wide, int* __restrict__ out)
 {
     long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    int m01 = 0, m18 = 0, m08 = 0, mw = 0;
+    int m01 = 0, m18 = 0, m08 = 0, mw = 0, mf = 0;
     if (c < B.ncell) {
         const Rep& rp = B.rep[B.rep_of_cell[c]];
         const int* st = start + rp.cell0;
@@ -141,6 +142,7 @@ __global__ void k_unit_max(Batch B, const int* __restrict__ start, int wide, int
             int k = st[nc + 1] - st[nc];
             m01 += k;
             if (t >= 13) m18 += k;
+            if (t >= 9) mf += k;
             if (dx >= 0 && dy >= 0 && dz >= 0) m08 += k;
         }
         // the wide traversal's 5^3 neighbourhood (only when that traversal is in use)
@@ -154,21 +156,23 @@ __global__ void k_unit_max(Batch B, const int* __restrict__ start, int wide, int
         m18 = max(m18, __shfl_down_sync(0xffffffffu, m18, o));
         m08 = max(m08, __shfl_down_sync(0xffffffffu, m08, o));
         mw = max(mw, __shfl_down_sync(0xffffffffu, mw, o));
+        mf = max(mf, __shfl_down_sync(0xffffffffu, mf, o));
     }
     // block maximum first: one global atomic per value and block
-    __shared__ int s_m[4][32];
+    __shared__ int s_m[5][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (lane == 0) {
         s_m[0][warp] = m01;
         s_m[1][warp] = m18;
         s_m[2][warp] = m08;
         s_m[3][warp] = mw;
+        s_m[4][warp] = mf;
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
+    if (threadIdx.x < 5) {
         int m = 0;
         for (int w = 0; w < nw; w++) m = max(m, s_m[threadIdx.x][w]);
-        atomicMax(out + threadIdx.x, m);
+        atomicMax(out + (threadIdx.x == 4 ? ATM_FWD_UNIT : (int)threadIdx.x), m);
         // the corner-anchored 3c08 stages the same blocks as 3c08
         if (threadIdx.x == 2) atomicMax(out + 4, m);
     }
@@ -536,6 +540,51 @@ __global__ void __launch_bounds__(128) k_rdf(Batch B, const double* __restrict__
 
 // ---------------------------------------------------------------- reductions
 
+// candidate triplets of the cell tasks of unit u (index inside its replica)
+// and its half-shell candidate pairs
+__device__ void cell_candidates(const Grid& g, const int* st, int trav, long long u,
+                                unsigned long long& c3, unsigned long long& c2)
+{
+    int cx, cy, cz;
+    cell_coords(g, u, cx, cy, cz);
+    auto C2 = [](unsigned long long m) { return m < 2 ? 0ull : m * (m - 1) / 2; };
+    auto C3 = [](unsigned long long m) { return m < 3 ? 0ull : m * (m - 1) * (m - 2) / 6; };
+    unsigned long long N[8];           // 3c08's block, by slot
+    unsigned long long before = 0, pairs = 0, one = 0, all = 0;  // 3c18: the forward cells so far
+    const unsigned long long N0 = (unsigned long long)(st[u + 1] - st[u]);
+#pragma unroll
+    for (int t = 0; t < 27; t++) {
+        const int dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
+        if (t < 13 && trav != 0) continue;
+        const long long c = cell_at(g, cx, cy, cz, dx, dy, dz);
+        const unsigned long long k = (unsigned long long)(st[c + 1] - st[c]);
+        all += k;
+        if (t > 13) {
+            pairs += k * before;
+            one += k * C2(N0) + N0 * C2(k);
+            before += k;
+        }
+        if (dx >= 0 && dy >= 0 && dz >= 0) N[dx + 2 * dy + 4 * dz] = k;
+    }
+    c2 += C2(N0) + N0 * before;
+    if (trav == 0) {
+        c3 += all > 0 ? N0 * C2(all - 1) : 0ull;
+    } else if (trav == 1) {
+        c3 += C3(N0) + one + N0 * pairs;
+    } else {
+        c3 += C3(N0);
+#pragma unroll
+        for (int s = 0; s < 8; s++)
+#pragma unroll
+            for (int t = s + 1; t < 8; t++) {
+                if ((s & t) == 0) c3 += N[t] * C2(N[s]) + N[s] * C2(N[t]);
+#pragma unroll
+                for (int v = t + 1; v < 8; v++)
+                    if ((s & t & v) == 0) c3 += N[s] * N[t] * N[v];
+            }
+    }
+}
+
 // Two-level reduction in a fixed order (the same sums for the same partials).  Level 1: CTA
 // (r, k) sums the k-th of REDUCE_PARTS equal slices of replica r's units and
 // molecules (thread-strided, then a fixed tree).  Level 2: one warp per
@@ -547,9 +596,10 @@ __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
     const int tid = threadIdx.x;
     const int r = blockIdx.x / REDUCE_PARTS, k = blockIdx.x % REDUCE_PARTS;
     const Rep& rp = R.b.rep[r];
-    const long long cu = (rp.g.ncell + REDUCE_PARTS - 1) / REDUCE_PARTS;
+    const long long nu = rp.g.ncell * R.split, uf = rp.cell0 * R.split;
+    const long long cu = (nu + REDUCE_PARTS - 1) / REDUCE_PARTS;
     const long long cm = (rp.n + REDUCE_PARTS - 1) / REDUCE_PARTS;
-    const long long u0 = rp.cell0 + k * cu, u1 = min(rp.cell0 + rp.g.ncell, u0 + cu);
+    const long long u0 = uf + k * cu, u1 = min(uf + nu, u0 + cu);
     const long long m0 = rp.mol0 + k * cm, m1 = min(rp.mol0 + rp.n, m0 + cm);
     double e3 = 0, w3 = 0, e2 = 0, w2 = 0, ke = 0;
     unsigned long long c3 = 0, i3 = 0, c2 = 0, v2 = 0;
@@ -564,6 +614,14 @@ __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
             c2 += R.unit_cnt2[2 * q];
             v2 += R.unit_cnt2[2 * q + 1];
         }
+    }
+    if (R.cand_trav >= 0) {
+        const long long cc = (rp.g.ncell + REDUCE_PARTS - 1) / REDUCE_PARTS;
+        const long long l1 = min(rp.g.ncell, (k + 1) * cc);
+        for (long long q = k * cc + tid; q < l1; q += 256)
+            if (unit_owned(rp, q))
+                cell_candidates(rp.g, R.cell_start + rp.cell0, R.cand_trav, q, c3, c2);
+        if (!R.unit_ew2) c2 = 0;  // (counted with the molecules below)
     }
     for (long long q = m0 + tid; q < m1; q += 256) {
         if (!R.unit_ew2) {
@@ -677,7 +735,7 @@ cudaError_t launch_build_cells(const Batch& b, double* x, int* cell_of, int* ran
     if (e != cudaSuccess) return e;
     if (n > 0) k_wrap_bin<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(b, x, cell_of, rank, count, status);
     k_scan<<<1, 1024, 0, st>>>(b.ncell, count, start, maxocc);
-    e = cudaMemsetAsync(maxocc + 1, 0, ATM_NTRAV * sizeof(int), st);
+    e = cudaMemsetAsync(maxocc + 1, 0, ATM_NUNIT * sizeof(int), st);
     if (e != cudaSuccess) return e;
     k_unit_max<<<nblk(b.ncell, MD_BLOCK), MD_BLOCK, 0, st>>>(b, start, wide ? 1 : 0, maxocc + 1);
     if (n > 0) {

@@ -34,6 +34,12 @@ struct ReduceArgs {
     // per unit ([2 ncell] each) replace mol_ew / mol_cnt
     const double* unit_ew2 = nullptr;
     const unsigned long long* unit_cnt2 = nullptr;
+    int split = 1;            // partial sums per cell of the unit arrays
+    // forward lists: the candidates of the cell tasks (traversal 0, 1 or 2) and
+    // of the half-shell pairs are counted here from the cells (-1: unit_cnt
+    // and unit_cnt2 hold them)
+    int cand_trav = -1;
+    const int* cell_start = nullptr;
     ResultDev* part;          // [R * REDUCE_PARTS] partial sums
     ResultDev* out;           // [R]
 };
@@ -44,7 +50,7 @@ constexpr int LJ_BLOCK = 128;
 constexpr int MD_BLOCK = 256;
 
 // maxocc[0] = largest cell occupancy, maxocc[1..5] = largest unit of 3c01, 3c18, 3c08, 3cw,
-// corner-anchored 3c08 (3cw's only when wide; 0 otherwise)
+// corner-anchored 3c08 (3cw's only when wide; 0 otherwise), maxocc[6] = of the forward lists
 cudaError_t launch_build_cells(const Batch& b, double* x, int* cell_of, int* rank, int* count,
                                int* start, int* perm, double* xl, float* xl32, int* cell_sorted,
                                int* maxocc, int* status, bool wide, cudaStream_t st);

@@ -32,7 +32,8 @@ constexpr size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct NaLayout {
     size_t rep, rep_of_cell, rep_of_mol, x, cell_of, rank, count, start, perm, cell_sorted, xl,
-        xl32, f_lj, f_atm, unit_ew, unit_cnt, mol_ew, mol_cnt, ke, res, status, maxocc, total;
+        xl32, f_lj, f_atm, unit_ew, unit_cnt, unit_ew2, unit_cnt2, mol_ew, mol_cnt, ke, res, status,
+        maxocc, total;
 };
 
 constexpr long long NA_N = ATM_NOALLOC_MAX_N;
@@ -58,18 +59,20 @@ constexpr NaLayout na_layout()
     L.f_atm = o;       o = al256(o + 3 * NA_N * sizeof(double));
     L.unit_ew = o;     o = al256(o + 2 * NA_C * sizeof(double));
     L.unit_cnt = o;    o = al256(o + 2 * NA_C * sizeof(unsigned long long));
+    L.unit_ew2 = o;    o = al256(o + 2 * NA_C * sizeof(double));
+    L.unit_cnt2 = o;   o = al256(o + 2 * NA_C * sizeof(unsigned long long));
     L.mol_ew = o;      o = al256(o + 2 * NA_N * sizeof(double));
     L.mol_cnt = o;     o = al256(o + 2 * NA_N * sizeof(unsigned));
     L.ke = o;          o = al256(o + NA_N * sizeof(double));
     L.res = o;         o = al256(o + (1 + REDUCE_PARTS) * sizeof(ResultDev));
     L.status = o;      o = al256(o + sizeof(int));
-    L.maxocc = o;      o = al256(o + (1 + ATM_NTRAV) * sizeof(int));
+    L.maxocc = o;      o = al256(o + (1 + ATM_NUNIT) * sizeof(int));
     L.total = o;
     return L;
 }
 constexpr NaLayout NA = na_layout();
 
-// the scratch array (about 6.7 MB at the limits above)
+// the scratch array (about 7.8 MB at the limits above)
 __device__ __align__(256) unsigned char g_na_scratch[NA.total];
 
 constexpr int NA_MAX_DEVICES = 64;
@@ -165,6 +168,8 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     double* f_atm = reinterpret_cast<double*>(base + NA.f_atm);
     double* unit_ew = reinterpret_cast<double*>(base + NA.unit_ew);
     unsigned long long* unit_cnt = reinterpret_cast<unsigned long long*>(base + NA.unit_cnt);
+    double* unit_ew2 = reinterpret_cast<double*>(base + NA.unit_ew2);
+    unsigned long long* unit_cnt2 = reinterpret_cast<unsigned long long*>(base + NA.unit_cnt2);
     double* mol_ew = reinterpret_cast<double*>(base + NA.mol_ew);
     unsigned* mol_cnt = reinterpret_cast<unsigned*>(base + NA.mol_cnt);
     double* ke = reinterpret_cast<double*>(base + NA.ke);
@@ -194,7 +199,7 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     if (n > 0) NA_CU(launch_check_finite(3 * n, x, status, st));
     NA_CU(launch_build_cells(b, x, cell_of, rank, count, start, perm, xl, xl32, cell_sorted,
                              maxocc, status, false, st));
-    int hocc[1 + ATM_NTRAV] = {}, hstat = 0;
+    int hocc[1 + ATM_NUNIT] = {}, hstat = 0;
     NA_CU(cudaMemcpyAsync(hocc, maxocc, sizeof(hocc), cudaMemcpyDeviceToHost, st));
     NA_CU(cudaMemcpyAsync(&hstat, status, sizeof(int), cudaMemcpyDeviceToHost, st));
     NA_CU(cudaStreamSynchronize(st));
@@ -225,7 +230,14 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     j.persistent = 0;
     j.nwarps = 0;
     j.st = st;
-    NA_CU(enqueue_lj(j));
+    j.unit_ew2 = unit_ew2;
+    j.unit_cnt2 = unit_cnt2;
+    j.mcap_fwd = std::max(1, hocc[1 + ATM_FWD_UNIT]);
+    j.whole = true;
+    j.lj_apart = true;
+    j.nruns = fwd_runs_of(rp.g);
+    const FwdLaunch fwd = atm_fwd_plan(j);
+    if (fwd.lj != 2) NA_CU(enqueue_lj(j));
     bool capacity = false;
     cudaError_t e = enqueue_atm(j, nullptr, &capacity);
     if (capacity) return ATM_E_CAPACITY;
@@ -238,6 +250,13 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     r.unit_cnt = unit_cnt;
     r.mol_ew = mol_ew;
     r.mol_cnt = mol_cnt;
+    if (fwd.lj == 2) {
+        r.unit_ew2 = unit_ew2;
+        r.unit_cnt2 = unit_cnt2;
+    }
+    r.split = fwd.use ? fwd.split : 1;
+    r.cand_trav = fwd.use ? (int)trav : -1;
+    r.cell_start = start;
     r.ke = ke;
     r.part = res + 1;
     r.out = res;

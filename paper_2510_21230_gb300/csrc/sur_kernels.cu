@@ -28,6 +28,17 @@ struct SurAcc {
 // one subtraction of an immediate, one square and one base-2 exponential.
 constexpr float SUR_SQH = 0.8493218002880191f;  // sqrt(log2(e) / 2)
 
+// compensated running sum
+struct Kahan {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float v)
+    {
+        const float y = __fsub_rn(v, c), t = __fadd_rn(s, y);
+        c = __fsub_rn(__fsub_rn(t, s), y);
+        s = t;
+    }
+};
+
 struct SurConst {
     float rc2, sg, sv, pi_rc;  // sg = s / d_g, sv = s / d_v
 };
@@ -158,7 +169,8 @@ __global__ void __launch_bounds__(SUR_BLOCK, 5) k_sur_desc(const SurForceArgs A)
         return __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
     };
     // LJ of one neighbour (the FP32 LJ kernel's expressions)
-    float ljx = 0.f, ljy = 0.f, ljz = 0.f, lje = 0.f, ljw = 0.f;
+    Kahan ljx, ljy, ljz;  // (plain sums of the 50 odd terms round at 1e-6 of the force)
+    float lje = 0.f, ljw = 0.f;
     unsigned lj_cand = 0u, lj_pairs = 0u;
     // fwd: the neighbour is in the forward half shell (a later molecule of the
     // own cell, or a forward cell), so the pair is counted once, here
@@ -168,9 +180,9 @@ __global__ void __launch_bounds__(SUR_BLOCK, 5) k_sur_desc(const SurForceArgs A)
         const float s3 = s2 * s2 * s2;
         const float s6 = s3 * s3;
         const float fw = (rp.eps48f * s6 - rp.eps24f * s3) * ia;
-        ljx -= fw * ex;
-        ljy -= fw * ey;
-        ljz -= fw * ez;
+        ljx.add(-(fw * ex));
+        ljy.add(-(fw * ey));
+        ljz.add(-(fw * ez));
         lje += rp.eps4f * (s6 - s3) - rp.ushiftf;
         ljw += fw * a;
         lj_pairs += fwd ? 1u : 0u;
@@ -244,9 +256,9 @@ __global__ void __launch_bounds__(SUR_BLOCK, 5) k_sur_desc(const SurForceArgs A)
         }
     }
     if (LJ) {
-        A.f_lj[s] = (double)ljx;
-        A.f_lj[n + s] = (double)ljy;
-        A.f_lj[2 * n + s] = (double)ljz;
+        A.f_lj[s] = (double)ljx.s;
+        A.f_lj[n + s] = (double)ljy.s;
+        A.f_lj[2 * n + s] = (double)ljz.s;
         A.mol_ew[2 * s] = 0.5 * (double)lje;
         A.mol_ew[2 * s + 1] = 0.5 * (double)ljw;
         A.mol_cnt[2 * s] = lj_cand;
