@@ -226,7 +226,7 @@ atm_status atm3::sur_enqueue_atm(atm_ctx* c)
     a.mol_cnt = c->mol_cnt;
     a.mode = 0;
     CU(launch_sur_forces(a, c->st));
-    c->n_launch += SUR_LAUNCHES;
+    c->n_launch += sur_launches(a);
     return ATM_OK;
 }
 
@@ -246,7 +246,7 @@ atm_status atm3::sur_enqueue_monitor(atm_ctx* c)
     a.mode = 0;
     CU(launch_sur_forces(a, c->st));
     CU(launch_sur_diff(c->n, S->f_scratch, c->f_atm, S->d_mon, c->st));
-    c->n_launch += SUR_LAUNCHES + 1;
+    c->n_launch += sur_launches(a) + 1;
     S->checks += 1;
     return ATM_OK;
 }
@@ -389,7 +389,7 @@ extern "C" atm_status atm_surrogate_descriptors(atm_ctx* c, float* desc, float* 
     a.row0 = 0;
     a.mode = 1;
     CU(launch_sur_forces(a, c->st));
-    c->n_launch += 2;  // packing + descriptors
+    c->n_launch += sur_launches(a) - 1;  // (packing and) descriptors
     std::vector<float> ds(n * SUR_ND), vs(n * SUR_NV);
     std::vector<int32_t> perm(n);
     CU(cudaMemcpyAsync(ds.data(), a.d_out, n * SUR_ND * 4, cudaMemcpyDeviceToHost, c->st));
@@ -597,7 +597,7 @@ extern "C" atm_status atm_surrogate_add_frame(atm_ctx* c, atm_traversal trav, at
     a.row0 = S->rows;
     a.mode = 1;
     CU(launch_sur_forces(a, c->st));
-    c->n_launch += 2;  // packing + descriptors
+    c->n_launch += sur_launches(a) - 1;  // (packing and) descriptors
     s = ctx_sync_and_check(c);
     if (s != ATM_OK) return s;
     S->rows += c->n;

@@ -134,8 +134,11 @@ struct SurAdamArgs {
     float lr, beta1, beta2, eps, c1, c2;  // c1 = 1 - beta1^t, c2 = 1 - beta2^t
 };
 
-// descriptors (and, mode 0, the MLP and the force): three launches
+// descriptors (and, mode 0, the MLP and the force): two launches, or three (with
+// packed coordinates) for large systems
 cudaError_t launch_sur_forces(const SurForceArgs& a, cudaStream_t st);
+bool sur_by_warps(const SurForceArgs& a);
+inline int sur_launches(const SurForceArgs& a) { return sur_by_warps(a) ? 2 : 3; }
 constexpr int SUR_LAUNCHES = 3;
 // MLP on given descriptor rows (no neighbour search): w[n][3], f[n][3]
 cudaError_t launch_sur_mlp_rows(long long n, const float* D, const float* V,
