@@ -274,6 +274,41 @@ __host__ __device__ inline FwdSmem fwd_smem_plan(int mcap, int run, int nwarps)
     return p;
 }
 
+// Arguments of the FP64 forward-list kernels (atm_list64.cu).  Per sorted
+// molecule i, rows of `stride` entries: its list (sorted index of the partner;
+// 18-cell slot | place in the partner's cell << 8) and the pair scalars of the
+// list's edges; per 18-cell slot the bitmap of the partners in that cell and
+// the list place of the first of them.
+struct List64Args {
+    Batch b;
+    long long n;              // SoA stride = b.ntot
+    const double* x;          // wrapped positions, original order, SoA [3n]
+    const int* perm;          // sorted -> original
+    const double* xl;         // sorted cell-local coordinates, FP64 and FP32
+    const float* xl32;
+    const int* cell_start;
+    const int* cell_sorted;
+    uint2* list;
+    double* G;
+    long long stride;
+    uint2* place;             // [18 n]
+    int* count;               // [n] list lengths
+    double* mol_w3;           // [n] W3 of the edges of a molecule's list
+    unsigned* mol_n3;         // [n] triplets whose lowest molecule it is
+    double* mol_ew;           // [2n] E2, W2 of its list
+    unsigned* mol_cnt;        // [2n] 0, pairs
+    double* fs;               // sorted-order force (zero at launch): ATM, or LJ + ATM (lj = 1)
+    double* fs_lj;            // lj = 2: the LJ force (zero at launch)
+    int* status;
+    int mcap;                 // molecule capacity of 18 cells (<= stride)
+    int run;                  // as FwdArgs
+    const int* runs;
+    long long nruns;
+    int split;
+    int lj;
+};
+constexpr size_t LIST64_SMEM = 96 << 10;  // most shared memory the list kernel takes
+
 // pair bitmaps: word k - 13 of molecule s (sorted) covers the molecules of
 // the cell at offset27(k), k = 13 (its own cell, the later molecules) .. 26
 // (the 13 forward cells); a cell holds at most PM_CELL_MAX molecules
@@ -499,6 +534,9 @@ cudaError_t launch_block_det64(int trav, int trunc, const AtmArgs<double>& a, in
                                size_t smem, int ctas, cudaStream_t s);
 cudaError_t launch_block_det32(int trav, int trunc, const AtmArgs<float>& a, int nwarps,
                                size_t smem, int ctas, cudaStream_t s);
+// the FP64 forward-list kernels (atm_list64.cu)
+cudaError_t launch_list64(const List64Args& a, cudaStream_t s);
+size_t list64_smem(int mcap, int run);
 // the forward-list kernel (atm_fwd.cu), one CTA of nwarps warps per cell and
 // part; the shared-memory limit is raised as needed
 cudaError_t launch_atm_fwd(const FwdArgs& a, int det, int nwarps, cudaStream_t s);

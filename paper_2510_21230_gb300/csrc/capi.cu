@@ -118,7 +118,8 @@ static void free_all(atm_ctx* c)
                    c->f_lj, c->f_atm, c->f_out, c->unit_ew, c->unit_cnt, c->mol_ew, c->mol_cnt,
                    c->ke, c->d_res, c->d_part, c->d_status, c->d_maxocc, c->d_work, c->d_dens,
                    c->d_rdf, c->d_ttarget, c->unit_ew2, c->unit_cnt2, c->f_in, c->d_chk,
-                   c->d_ulist, c->d_ucount, c->d_runs, c->pmask};
+                   c->d_ulist, c->d_ucount, c->d_runs, c->pmask, c->l64.list, c->l64.G, c->l64.place,
+                   c->l64.count, c->l64.mol_w3, c->l64.mol_n3};
     for (void* p : dev)
         if (p) cudaFree(p);
     if (c->h_res) cudaFreeHost(c->h_res);
@@ -557,7 +558,8 @@ static bool fwd_active(const atm_ctx* c, int trav, int trunc, int prec)
     j.mcap_fwd = graph_mcap_fwd(c);
     j.runs = c->d_runs;
     j.nruns = c->nruns;
-    return atm_fwd_plan(j).use;
+    j.l64 = c->maxocc <= PM_CELL_MAX ? &c->l64 : nullptr;
+    return atm_uses_lists(j);
 }
 
 static void launch_choice(atm_ctx* c, int trav, int trunc, int prec, int mcap, int& persistent,
@@ -618,6 +620,42 @@ static bool use_pair_masks(const atm_ctx* c, int trav, int trunc, int prec)
     return c->opt_pmask && c->pmask && prec == ATM_FP32C && trunc == ATM_TRUNC_PAIR &&
            (trav == ATM_3C08 || trav == ATM_3C08A || (trav == ATM_3C18 && c->pm_3c18)) &&
            c->maxocc <= atm3::PM_CELL_MAX;
+}
+
+void atm3::ctx_want_list64(atm_ctx* c, int trav, int trunc, int prec, int mcap)
+{
+    if (prec != ATM_FP64 || trunc != ATM_TRUNC_PAIR || (trav != ATM_3C01 && trav != ATM_3C18 && trav != ATM_3C08) ||
+        c->det || !c->whole || c->n <= 0 || c->maxocc > PM_CELL_MAX)
+        return;
+    List64Args& l = c->l64;
+    if (l.list && l.stride >= mcap) return;
+    // a row for any list of an 18-cell unit, with room for units to grow
+    const long long stride = ((mcap + mcap / 8 + 15) / 8) * 8;
+    const size_t rows = (size_t)c->n * (size_t)stride;
+    cudaStreamSynchronize(c->st);
+    drop_graph(c);
+    void* old[] = {l.list, l.G, l.place, l.count, l.mol_w3, l.mol_n3};
+    for (void* p : old)
+        if (p) cudaFree(p);
+    l = List64Args{};
+    if (rows * 16 > ((size_t)16 << 30)) return;  // (the block kernel then)
+    bool ok = cudaMalloc((void**)&l.list, rows * sizeof(uint2)) == cudaSuccess;
+    ok = ok && cudaMalloc((void**)&l.G, (rows + PM_CELL_MAX) * sizeof(double)) == cudaSuccess;
+    ok = ok && cudaMalloc((void**)&l.place, 18 * (size_t)c->n * sizeof(uint2)) == cudaSuccess;
+    ok = ok && cudaMalloc((void**)&l.count, (size_t)c->n * sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMalloc((void**)&l.mol_w3, (size_t)c->n * sizeof(double)) == cudaSuccess;
+    ok = ok && cudaMalloc((void**)&l.mol_n3, (size_t)c->n * sizeof(unsigned)) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        void* got[] = {l.list, l.G, l.place, l.count, l.mol_w3, l.mol_n3};
+        for (void* p : got)
+            if (p) cudaFree(p);
+        l = List64Args{};
+        return;
+    }
+    l.stride = stride;
+    l.x = c->x;
+    l.perm = c->perm;
 }
 
 // LJ + ATM force kernels for the current cells; mcap = staged-molecule capacity
@@ -686,10 +724,12 @@ atm_status atm3::ctx_enqueue_forces(atm_ctx* c, int trav, int trunc, int prec, i
     j.lj_apart = prec != ATM_SURROGATE && !fused;
     j.runs = c->d_runs;
     j.nruns = c->nruns;
-    const FwdLaunch fwd = atm_fwd_plan(j);
+    if (!c->capturing) ctx_want_list64(c, trav, trunc, prec, j.mcap_fwd);
+    j.l64 = c->maxocc <= PM_CELL_MAX ? &c->l64 : nullptr;
+    const FwdLaunch fwd = atm_fwd_plan(j), l64 = atm_list64_plan(j);
 
     cudaEvent_t ev;
-    if (prec != ATM_SURROGATE && !fused && fwd.lj != 2) {
+    if (prec != ATM_SURROGATE && !fused && fwd.lj != 2 && !l64.use) {
         // (the surrogate's descriptor pass computes LJ from the same neighbours)
         ev = ctx_prof_begin(c, PK_LJ);
         CU(enqueue_lj(j));
@@ -723,9 +763,11 @@ atm_status atm3::ctx_enqueue_forces(atm_ctx* c, int trav, int trunc, int prec, i
     c->f_trunc = trunc;
     c->f_prec = prec;
     c->f_fused = fused;
-    c->f_unit_lj = fused || (fwd.use && fwd.lj == 2);
+    if (l64.use) c->n_launch += 2;  // lists, triangles and edges
+    c->f_unit_lj = (fused && !l64.use) || (fwd.use && fwd.lj == 2);
     c->f_split = fwd.use ? fwd.split : 1;
-    c->f_fwd = fwd.use;
+    c->f_fwd = fwd.use || l64.use;
+    c->f_l64 = l64.use;
     return ATM_OK;
 }
 
@@ -740,6 +782,11 @@ static atm_status enqueue_reduce(atm_ctx* c)
     r.split = c->f_split;
     r.cand_trav = c->f_fwd ? c->f_trav : -1;
     r.cell_start = c->start;
+    if (c->f_l64) {
+        r.mol_w3 = c->l64.mol_w3;
+        r.mol_n3 = c->l64.mol_n3;
+        r.visits = c->f_trav == ATM_3C01 ? 3 : 1;  // 3c01 counts owner visits
+    }
     r.mol_ew = c->mol_ew;
     r.mol_cnt = c->mol_cnt;
     r.ke = c->ke;
@@ -933,6 +980,7 @@ static atm_status run_graph_steps(atm_ctx* c, int nsteps, int trav, int trunc, i
     int persistent = 0, nwarps = 0, cls[3] = {1, 0, 0};
     if (prec != ATM_SURROGATE)
         launch_choice(c, trav, trunc, prec, c->unit_max[trav], persistent, nwarps, cls);
+    ctx_want_list64(c, trav, trunc, prec, graph_mcap_fwd(c));
     const bool fwd = fwd_active(c, trav, trunc, prec);
     if (fwd) cls[0] = 1;
     const int mcap = graph_mcap(c, trav, trunc, prec, nwarps);
@@ -948,7 +996,9 @@ static atm_status run_graph_steps(atm_ctx* c, int nsteps, int trav, int trunc, i
         c->st = c->cap_st;
         cudaGraph_t g = nullptr;
         CU(cudaStreamBeginCapture(c->cap_st, cudaStreamCaptureModeThreadLocal));
+        c->capturing = true;
         atm_status s = enqueue_step(c, trav, trunc, prec, mcap);
+        c->capturing = false;
         cudaError_t e = cudaStreamEndCapture(c->cap_st, &g);
         c->st = keep;
         c->prof = keep_prof;
@@ -967,7 +1017,7 @@ static atm_status run_graph_steps(atm_ctx* c, int nsteps, int trav, int trunc, i
     cudaEvent_t ev = ctx_prof_begin(c, PK_MD);
     for (int k = 0; k < nsteps; k++) CU(cudaGraphLaunch(c->graph, c->st));
     ctx_prof_end(c, PK_MD, ev);
-    c->n_launch += (long long)nsteps * kernels_per_step(trav, trunc, prec, cls[0]);
+    c->n_launch += (long long)nsteps * (kernels_per_step(trav, trunc, prec, cls[0]) + (c->f_l64 ? 2 : 0));
     c->n_atm += nsteps;
     return ATM_OK;
 }

@@ -83,6 +83,8 @@ struct atm_ctx {
     bool f_unit_lj = false;  // the LJ sums of the current forces are in unit_ew2 / unit_cnt2
     int f_split = 1;         // partial sums per cell in the unit arrays
     bool f_fwd = false;      // the current forces came from forward lists
+    bool f_l64 = false;      // and those were the FP64 ones
+    atm3::List64Args l64{};  // their buffers (first used: allocated)
     bool whole = true;       // every replica owns all its layers
     bool wide_cells = false;  // cell builds also size the wide traversal's 5^3 units
     // forces of the current state given by the caller (original order, total),
@@ -121,6 +123,7 @@ struct atm_ctx {
     cudaEvent_t ev_io = nullptr, ev_io_done = nullptr;
     double* x_host_out = nullptr;  // where the last step copies its positions early
     bool x_out_issued = false;     // that copy is in flight on io_st
+    bool capturing = false;  // a step is being captured: nothing may be allocated
     cudaGraphExec_t graph = nullptr;
     int graph_key[10] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
     // profiling: event pairs around launch groups, summed per kind
@@ -155,6 +158,10 @@ atm_status ctx_enqueue_forces(atm_ctx* c, int trav, int trunc, int prec, int mca
 // profiling of a launch group (kind: 0 cells, 1 LJ, 2 ATM, 3 MD)
 cudaEvent_t ctx_prof_begin(atm_ctx* c, int kind);
 void ctx_prof_end(atm_ctx* c, int kind, cudaEvent_t a);
+
+// buffers of the FP64 forward lists for units of mcap molecules, if they can be
+// had (called outside stream captures)
+void ctx_want_list64(atm_ctx* c, int trav, int trunc, int prec, int mcap);
 
 // surrogate hooks (sur_capi.cu)
 atm_status sur_enqueue_atm(atm_ctx* c);       // surrogate force into f_atm; unit sums zeroed

@@ -78,6 +78,9 @@ struct ForceJob {
     int mcap_fwd = 0;
     bool whole = false;
     bool lj_apart = false;
+    // FP64 pair rule from forward lists (atm_list64.cu): the buffers and inputs
+    // of List64Args (list nullptr: not taken), cells within PM_CELL_MAX
+    const List64Args* l64 = nullptr;
     const int* runs = nullptr;  // FwdArgs.runs and nruns of FWD_RUN cells (device)
     long long nruns = 0;
 };
@@ -89,6 +92,13 @@ struct FwdLaunch {
     int nwarps = FWD_MAXW, run = FWD_RUN, split = 1;
 };
 FwdLaunch atm_fwd_plan(const ForceJob& j);
+// the same for the FP64 lists (lj 1 or 2)
+FwdLaunch atm_list64_plan(const ForceJob& j);
+// either
+inline bool atm_uses_lists(const ForceJob& j)
+{
+    return atm_fwd_plan(j).use || atm_list64_plan(j).use;
+}
 // runs of FWD_RUN cells of one replica's grid
 inline long long fwd_runs_of(const Grid& g)
 {

@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
     const long long m0 = rp.mol0 + k * cm, m1 = min(rp.mol0 + rp.n, m0 + cm);
     double e3 = 0, w3 = 0, e2 = 0, w2 = 0, ke = 0;
     unsigned long long c3 = 0, i3 = 0, c2 = 0, v2 = 0;
-    for (long long q = u0 + tid; q < u1; q += 256) {
+    for (long long q = u0 + tid; q < u1 && !R.mol_w3; q += 256) {
         e3 += R.unit_ew[2 * q];
         w3 += R.unit_ew[2 * q + 1];
         c3 += R.unit_cnt[2 * q];
@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
         for (long long q = k * cc + tid; q < l1; q += 256)
             if (unit_owned(rp, q))
                 cell_candidates(rp.g, R.cell_start + rp.cell0, R.cand_trav, q, c3, c2);
-        if (!R.unit_ew2) c2 = 0;  // (counted with the molecules below)
+        if (!R.unit_ew2 && !R.mol_w3) c2 = 0;  // (counted with the molecules below)
     }
     for (long long q = m0 + tid; q < m1; q += 256) {
         if (!R.unit_ew2) {
@@ -630,8 +630,13 @@ __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
             c2 += R.mol_cnt[2 * q];
             v2 += R.mol_cnt[2 * q + 1];
         }
+        if (R.mol_w3) {
+            w3 += R.mol_w3[q];
+            i3 += (unsigned long long)R.visits * R.mol_n3[q];
+        }
         ke += R.ke[q];
     }
+    if (R.mol_w3) e3 = w3 / 9.0;  // u is homogeneous of degree -9 in the distances
     sd[0][tid] = e2; sd[1][tid] = e3; sd[2][tid] = w2; sd[3][tid] = w3; sd[4][tid] = ke;
     su[0][tid] = c3; su[1][tid] = i3; su[2][tid] = c2; su[3][tid] = v2;
     __syncthreads();

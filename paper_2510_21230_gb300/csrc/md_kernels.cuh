@@ -40,6 +40,11 @@ struct ReduceArgs {
     // and unit_cnt2 hold them)
     int cand_trav = -1;
     const int* cell_start = nullptr;
+    // FP64 forward lists: W3 (E3 = W3 / 9) and triplets per molecule instead of
+    // unit_ew and unit_cnt (nullptr: those); visits: owners that count a triplet
+    const double* mol_w3 = nullptr;
+    const unsigned* mol_n3 = nullptr;
+    int visits = 1;
     ResultDev* part;          // [R * REDUCE_PARTS] partial sums
     ResultDev* out;           // [R]
 };
