@@ -439,9 +439,10 @@ namespace {
 
 // gradient of the current master parameters over `batch` rows of (D, V, T)
 // (idx = nullptr: rows 0..batch-1); Adam step when update != 0
+// (sample > 0, tensor cores: the rows are drawn in the kernel from that many)
 atm_status grad_step(atm_ctx* c, SurState* S, const float* D, const float* V, const float* T,
                      const long long* idx, long long batch, double sigma2, int update, double lr,
-                     double* loss_dev, float* grad_dev)
+                     double* loss_dev, float* grad_dev, long long sample = 0, uint64_t seed = 0)
 {
     const int nct = S->train_tc ? sur_grad_tc_tiles(batch) : (int)((batch + SUR_TILE - 1) / SUR_TILE);
     if (nct > S->part_cap) {
@@ -460,6 +461,9 @@ atm_status grad_step(atm_ctx* c, SurState* S, const float* D, const float* V, co
     g.T = T;
     g.idx = idx;
     g.batch = batch;
+    g.S = sample;
+    g.seed = seed;
+    g.step = S->adam_t;
     g.P = S->P;
     g.mean = S->mean;
     g.scale = S->scale;
@@ -687,12 +691,12 @@ extern "C" atm_status atm_surrogate_train(atm_ctx* c, int64_t steps, int64_t bat
         S->loss_cap = steps;
     }
     for (long long t = 0; t < steps; t++) {
-        if (!full) {
+        if (!full && !S->train_tc) {
             CU(launch_sur_sample(S->idx, B, S->rows, seed, S->adam_t, c->st));
             c->n_launch += 1;
         }
         atm_status s = grad_step(c, S, S->D, S->V, S->T, full ? nullptr : S->idx, B, S->sigma2, 1,
-                                 lr, S->d_loss + t, nullptr);
+                                 lr, S->d_loss + t, nullptr, full || !S->train_tc ? 0 : S->rows, seed);
         if (s != ATM_OK) return s;
     }
     if (loss) CU(cudaMemcpyAsync(loss, S->d_loss, (size_t)steps * sizeof(double), cudaMemcpyDeviceToHost, c->st));

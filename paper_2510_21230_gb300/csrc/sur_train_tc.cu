@@ -3,8 +3,13 @@
 // tcgen05.mma with bfloat16 operands in shared memory and FP32 accumulators
 // in tensor memory (TMEM); FP32 master weights, FP32 gradients.
 //
-// One CTA of 128 threads per 128-sample tile (persistent over tiles); thread
-// t owns sample t and TMEM lane t.  Per tile:
+// One CTA of 512 threads per 128-sample tile (persistent over tiles); the four
+// threads t, t + 128, .. share sample t and TMEM lane t, a quarter of the columns
+// of every layer each.  A step of 8,192 samples has 64 tiles, fewer than SMs, so
+// the tile's chain of latencies bounds it: 46 us a step with one thread per
+// sample, 39 with four, 22 with rows, weights and gradients moved 16 bytes at a
+// time and the vectors fetched beside the first layers (their rows are random
+// lines of the data set).  Per tile:
 //   forward   Z1 = X W1, H1 = silu(Z1 + b1); Z2 = H1 W2, H2 = silu(Z2 + b2);
 //             w = H2 W3 + b3 (the inference kernel's arithmetic: bfloat16
 //             inputs, weights and hidden activations), F = sum_m w_m v_m
@@ -41,6 +46,8 @@ namespace {
 using namespace tc;
 
 constexpr int TR_M = 128;             // samples per tile = TMEM lanes
+constexpr int TR_T = 512;             // threads: four per sample
+constexpr int TR_VS = SUR_NV + 4;     // row stride of the staged vectors (16-byte reads without conflicts)
 constexpr uint32_t TR_COLS = 256;     // TMEM columns per CTA
 constexpr uint32_t SBO_K32 = 4 * 128, SBO_K64 = 8 * 128, SBO_K128 = 16 * 128;
 
@@ -57,6 +64,7 @@ struct TrSmem {
     alignas(128) unsigned char dyt[16 * TR_M * 2];  // B of dW3: N 16 (dL/dw_m) x K samples
     alignas(128) unsigned char dz2t[64 * TR_M * 2]; // B of dW2: N 64 x K samples
     alignas(128) unsigned char dz1t[64 * TR_M * 2]; // B of dW1: N 64 x K samples
+    alignas(16) float v[TR_M * TR_VS];              // the samples' vectors
     float w3[SUR_NH * SUR_NO];                      // FP32 master W3
     float b1[64], b2[64], b3[SUR_NO];
     double lsum[TR_M / 32];
@@ -73,6 +81,15 @@ __device__ __forceinline__ void put_bf(unsigned char* base, int row, int k, int 
         __float2bfloat16_rn(v);
 }
 
+// 16 floats to a 16-byte aligned row
+__device__ __forceinline__ void store16(float* to, const float (&o)[16])
+{
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+        reinterpret_cast<float4*>(to)[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+}
+static_assert(SUR_OFF_W1 % 4 == 0 && SUR_OFF_W2 % 4 == 0 && SUR_OFF_W3 % 4 == 0 && SUR_NP % 4 == 0, "rows of store16");
+
 // sigmoid and silu'(z) = s (1 + z (1 - s)); silu itself as the inference kernel forms it
 __device__ __forceinline__ float sigm(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
 
@@ -80,51 +97,56 @@ __device__ __forceinline__ float sigm(float z) { return __fdividef(1.0f, 1.0f + 
 
 namespace {
 
-__global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
+__global__ void __launch_bounds__(TR_T) k_sur_grad_tc(const SurGradArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
     TrSmem& S = *reinterpret_cast<TrSmem*>(smraw);
     const int tid = threadIdx.x, warp = tid >> 5;
+    const int t = tid & (TR_M - 1), part = tid / TR_M;  // sample, quarter of the columns
     const SurPacked* model = A.packed;
 
     // ---- once per CTA: weights, constant rows of the padded operands, barrier, TMEM
-    for (int e = tid; e < 64 * 4; e += TR_M) {
+    for (int e = tid; e < 64 * 4; e += TR_T) {
         const int r = e >> 2, j = e & 3;
         put_chunk(S.w1t, r, j, 4, *reinterpret_cast<const uint4*>(model->w1t + r * SUR_XS + 8 * j));
     }
-    for (int e = tid; e < 64 * 8; e += TR_M) {
+    for (int e = tid; e < 64 * 8; e += TR_T) {
         const int r = e >> 3, j = e & 7;
         put_chunk(S.w2t, r, j, 8, *reinterpret_cast<const uint4*>(model->w2t + r * SUR_HS + 8 * j));
     }
-    for (int e = tid; e < 16 * 8; e += TR_M) {
+    for (int e = tid; e < 16 * 8; e += TR_T) {
         const int r = e >> 3, j = e & 7;
         const uint4 z = make_uint4(0u, 0u, 0u, 0u);
         put_chunk(S.w3t, r, j, 8, r < SUR_NO ? *reinterpret_cast<const uint4*>(model->w3t + r * SUR_HS + 8 * j) : z);
     }
     // W2 itself (row k holds W2[k][j], j contiguous) for dH1 = dZ2 W2^T
-    for (int e = tid; e < SUR_NH * SUR_NH; e += TR_M)
-        put_bf(S.w2, e >> 6, e & 63, 8, A.P[SUR_OFF_W2 + e]);
-    for (int e = tid; e < SUR_NH * SUR_NO; e += TR_M) S.w3[e] = A.P[SUR_OFF_W3 + e];
+    for (int e = tid; e < 64 * 8; e += TR_T) {
+        const float4* w = reinterpret_cast<const float4*>(A.P + SUR_OFF_W2 + 8 * e);
+        const float4 a = w[0], b = w[1];
+        put_chunk(S.w2, e >> 3, e & 7, 8, make_uint4(pack_bf2(a.x, a.y), pack_bf2(a.z, a.w),
+                                                     pack_bf2(b.x, b.y), pack_bf2(b.z, b.w)));
+    }
+    for (int e = tid; e < SUR_NH * SUR_NO; e += TR_T) S.w3[e] = A.P[SUR_OFF_W3 + e];
     if (tid < 64) {
         S.b1[tid] = model->b1[tid];
         S.b2[tid] = model->b2[tid];
     }
     if (tid < SUR_NO) S.b3[tid] = model->b3[tid];
     {
-        // zero rows of the padded left operands
+        // zero rows of the padded left operands: beyond the weight rows (a group of
+        // 8 rows takes 2048 bytes)
         const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-        for (int e = tid; e < (int)(sizeof(S.xt) / 16); e += TR_M) {
-            reinterpret_cast<uint4*>(S.xt)[e] = z;
-            reinterpret_cast<uint4*>(S.h1t)[e] = z;
-            reinterpret_cast<uint4*>(S.h2t)[e] = z;
+        for (int e = tid; e < 12 * 128; e += TR_T) reinterpret_cast<uint4*>(S.xt + 4 * 2048)[e] = z;
+        for (int e = tid; e < 8 * 128; e += TR_T) {
+            reinterpret_cast<uint4*>(S.h1t + 8 * 2048)[e] = z;
+            reinterpret_cast<uint4*>(S.h2t + 8 * 2048)[e] = z;
         }
-        for (int e = tid; e < (int)(sizeof(S.dyt) / 16); e += TR_M) reinterpret_cast<uint4*>(S.dyt)[e] = z;
     }
     __syncthreads();
     // the rows of ones: their output rows are the bias gradients
-    put_bf(S.xt, SUR_ND, tid, 16, 1.0f);
-    put_bf(S.h1t, SUR_NH, tid, 16, 1.0f);
-    put_bf(S.h2t, SUR_NH, tid, 16, 1.0f);
+    if (part == 0) put_bf(S.xt, SUR_ND, t, 16, 1.0f);
+    if (part == 1) put_bf(S.h1t, SUR_NH, t, 16, 1.0f);
+    if (part == 2) put_bf(S.h2t, SUR_NH, t, 16, 1.0f);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&S.mbar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -141,7 +163,7 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem_base;
-    const uint32_t lane = tmem + ((uint32_t)(warp * 32) << 16);  // this warp's lane quarter
+    const uint32_t lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);  // this warp's lane quarter
     const uint32_t id64 = idesc_bf16(TR_M, 64), id16 = idesc_bf16(TR_M, 16);
 
     uint32_t phase = 0u;
@@ -169,28 +191,42 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
 
     const long long ntiles = (A.batch + TR_M - 1) / TR_M;
     for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const long long row = tile * TR_M + tid;
+        const long long row = tile * TR_M + t;
         const bool active = row < A.batch;
-        const long long smp = active ? (A.idx ? A.idx[row] : row) : 0;
+        const long long smp = !active ? 0 : (A.S > 0 ? sur_sample(A.seed, A.step, row, A.S)
+                                                     : (A.idx ? A.idx[row] : row));
 
         // ---- inputs: normalised descriptors (X and X^T), vectors, target
         {
-            float xv[SUR_ND];
+            float xv[8];
+            const int q0 = 8 * part;
+            const float4* drow = reinterpret_cast<const float4*>(A.D + smp * SUR_ND + q0);
+            const float4 d0 = drow[0], d1 = drow[1];
+            const float dv[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
 #pragma unroll
-            for (int q = 0; q < SUR_ND; q++)
-                xv[q] = active ? (A.D[smp * SUR_ND + q] - A.mean[q]) / A.scale[q] : 0.0f;
+            for (int q = 0; q < 8; q++)
+                xv[q] = active ? (dv[q] - A.mean[q0 + q]) / A.scale[q0 + q] : 0.0f;
+            put_chunk(S.x, t, part, 4, make_uint4(pack_bf2(xv[0], xv[1]), pack_bf2(xv[2], xv[3]),
+                                                  pack_bf2(xv[4], xv[5]), pack_bf2(xv[6], xv[7])));
 #pragma unroll
-            for (int j = 0; j < 4; j++)
-                put_chunk(S.x, tid, j, 4,
-                          make_uint4(pack_bf2(xv[8 * j], xv[8 * j + 1]), pack_bf2(xv[8 * j + 2], xv[8 * j + 3]),
-                                     pack_bf2(xv[8 * j + 4], xv[8 * j + 5]), pack_bf2(xv[8 * j + 6], xv[8 * j + 7])));
-#pragma unroll
-            for (int q = 0; q < SUR_ND; q++) put_bf(S.xt, q, tid, 16, xv[q]);
+            for (int q = 0; q < 8; q++) put_bf(S.xt, q0 + q, t, 16, xv[q]);
         }
         float tg[3];
 #pragma unroll
         for (int c = 0; c < 3; c++) tg[c] = active ? A.T[smp * 3 + c] : 0.0f;
-        const float* vrow = A.V + smp * SUR_NV;  // the sample's 16 vectors (read when active)
+        // the sample's 16 vectors to shared memory, 16 bytes at a time, beside the
+        // first two layers (read row by row from global memory in the loss they took
+        // 32 k of the tile's 66 k cycles)
+        {
+            const float* v = A.V + smp * SUR_NV + 12 * part;
+#pragma unroll
+            for (int q = 0; q < 3; q++)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(S.v + t * TR_VS + 12 * part + 4 * q)),
+                             "l"(v + 4 * q)
+                             : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
+        const float* vrow = S.v + t * TR_VS;
         publish();
 
         // ---- layer 1: TMEM [0, 64) = X W1
@@ -202,8 +238,8 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
         wait_mma();
         if (!ok) break;
         // H1 = silu(Z1 + b1) into the layer-2 operand and H1^T; silu'(Z1) to TMEM [160, 224)
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
+        {
+            const int q = part;
             float z[16], d[16];
             tmem_ld16(lane + 16 * q, z);
             uint32_t p[8];
@@ -213,12 +249,12 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
                 const float zb = z[i] + S.b1[k], s = sigm(zb);
                 d[i] = s * (1.0f + zb * (1.0f - s));
                 z[i] = silu(zb);
-                put_bf(S.h1t, k, tid, 16, z[i]);
+                put_bf(S.h1t, k, t, 16, z[i]);
             }
 #pragma unroll
             for (int i = 0; i < 8; i++) p[i] = pack_bf2(z[2 * i], z[2 * i + 1]);
-            put_chunk(S.h, tid, 2 * q, 8, make_uint4(p[0], p[1], p[2], p[3]));
-            put_chunk(S.h, tid, 2 * q + 1, 8, make_uint4(p[4], p[5], p[6], p[7]));
+            put_chunk(S.h, t, 2 * q, 8, make_uint4(p[0], p[1], p[2], p[3]));
+            put_chunk(S.h, t, 2 * q + 1, 8, make_uint4(p[4], p[5], p[6], p[7]));
             tmem_st16(lane + 160 + 16 * q, d);
         }
         publish();
@@ -232,8 +268,8 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
         wait_mma();
         if (!ok) break;
         // H2 (over H1: layer 2 has read it), H2^T; silu'(Z2) to TMEM [0, 64)
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
+        {
+            const int q = part;
             float z[16], d[16];
             tmem_ld16(lane + 64 + 16 * q, z);
             uint32_t p[8];
@@ -243,15 +279,17 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
                 const float zb = z[i] + S.b2[k], s = sigm(zb);
                 d[i] = s * (1.0f + zb * (1.0f - s));
                 z[i] = silu(zb);
-                put_bf(S.h2t, k, tid, 16, z[i]);
+                put_bf(S.h2t, k, t, 16, z[i]);
             }
 #pragma unroll
             for (int i = 0; i < 8; i++) p[i] = pack_bf2(z[2 * i], z[2 * i + 1]);
-            put_chunk(S.h, tid, 2 * q, 8, make_uint4(p[0], p[1], p[2], p[3]));
-            put_chunk(S.h, tid, 2 * q + 1, 8, make_uint4(p[4], p[5], p[6], p[7]));
+            put_chunk(S.h, t, 2 * q, 8, make_uint4(p[0], p[1], p[2], p[3]));
+            put_chunk(S.h, t, 2 * q + 1, 8, make_uint4(p[4], p[5], p[6], p[7]));
             tmem_st16(lane + 16 * q, d);
         }
         publish();
+
+        asm volatile("cp.async.wait_group 0;" ::: "memory");  // (ordered by wait_mma's barrier)
 
         // ---- layer 3: TMEM [128, 144) = H2 W3
         if (tid == 0) {
@@ -270,11 +308,12 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
 #pragma unroll
             for (int c = 0; c < 3; c++) {
                 float fc = 0.0f;
-                if (active)
+                if (active) {
 #pragma unroll
                     for (int m = 0; m < SUR_NO; m++) fc = fmaf(o[m] + S.b3[m], vrow[3 * m + c], fc);
+                }
                 r[c] = fc - tg[c];
-                loss += (double)r[c] * (double)r[c];
+                if (part == 0) loss += (double)r[c] * (double)r[c];
             }
             loss *= (double)A.norm;
             const float two_norm = 2.0f * A.norm;
@@ -283,12 +322,12 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
                 dy[m] = active ? two_norm * (r[0] * vrow[3 * m] + r[1] * vrow[3 * m + 1] +
                                              r[2] * vrow[3 * m + 2])
                                : 0.0f;
-                put_bf(S.dyt, m, tid, 16, dy[m]);
+                if ((m >> 2) == part) put_bf(S.dyt, m, t, 16, dy[m]);
             }
         }
         // dZ2 = (dY W3^T) silu'(Z2) over H2 (layer 3 has read it) and into dZ2^T
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
+        {
+            const int q = part;
             float s2[16], dz[16];
             tmem_ld16(lane + 16 * q, s2);
             uint32_t p[8];
@@ -299,12 +338,12 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
 #pragma unroll
                 for (int m = 0; m < SUR_NO; m++) dh = fmaf(dy[m], S.w3[SUR_NO * k + m], dh);
                 dz[i] = dh * s2[i];
-                put_bf(S.dz2t, k, tid, 16, dz[i]);
+                put_bf(S.dz2t, k, t, 16, dz[i]);
             }
 #pragma unroll
             for (int i = 0; i < 8; i++) p[i] = pack_bf2(dz[2 * i], dz[2 * i + 1]);
-            put_chunk(S.h, tid, 2 * q, 8, make_uint4(p[0], p[1], p[2], p[3]));
-            put_chunk(S.h, tid, 2 * q + 1, 8, make_uint4(p[4], p[5], p[6], p[7]));
+            put_chunk(S.h, t, 2 * q, 8, make_uint4(p[0], p[1], p[2], p[3]));
+            put_chunk(S.h, t, 2 * q + 1, 8, make_uint4(p[4], p[5], p[6], p[7]));
         }
         publish();
 
@@ -319,31 +358,31 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
         wait_mma();
         if (!ok) break;
         // dZ1 = dH1 silu'(Z1) into dZ1^T
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
+        {
+            const int q = part;
             float dh[16], s1[16];
             tmem_ld16(lane + 16 * q, dh);
             tmem_ld16(lane + 160 + 16 * q, s1);
 #pragma unroll
-            for (int i = 0; i < 16; i++) put_bf(S.dz1t, 16 * q + i, tid, 16, dh[i] * s1[i]);
+            for (int i = 0; i < 16; i++) put_bf(S.dz1t, 16 * q + i, t, 16, dh[i] * s1[i]);
         }
         // gradient rows of layers 3 and 2 (TMEM lane = output row)
         float* G = A.part + tile * SUR_NP;
-        {
+        if (part == 0) {
             float o[16];
             tmem_ld16(lane + 144, o);
-            if (tid < SUR_NH)
-                for (int m = 0; m < SUR_NO; m++) G[SUR_OFF_W3 + tid * SUR_NO + m] = o[m];
-            else if (tid == SUR_NH)
+            if (t < SUR_NH)
+                store16(G + SUR_OFF_W3 + t * SUR_NO, o);
+            else if (t == SUR_NH)
                 for (int m = 0; m < SUR_NO; m++) G[SUR_OFF_B3 + m] = o[m];
         }
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
+        {
+            const int q = part;
             float o[16];
             tmem_ld16(lane + 64 + 16 * q, o);
-            if (tid < SUR_NH)
-                for (int i = 0; i < 16; i++) G[SUR_OFF_W2 + tid * SUR_NH + 16 * q + i] = o[i];
-            else if (tid == SUR_NH)
+            if (t < SUR_NH)
+                store16(G + SUR_OFF_W2 + t * SUR_NH + 16 * q, o);
+            else if (t == SUR_NH)
                 for (int i = 0; i < 16; i++) G[SUR_OFF_B2 + 16 * q + i] = o[i];
         }
         publish();
@@ -356,18 +395,20 @@ __global__ void __launch_bounds__(TR_M) k_sur_grad_tc(const SurGradArgs A)
         }
         wait_mma();
         if (!ok) break;
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
+        {
+            const int q = part;
             float o[16];
             tmem_ld16(lane + 160 + 16 * q, o);
-            if (tid < SUR_ND)
-                for (int i = 0; i < 16; i++) G[SUR_OFF_W1 + tid * SUR_NH + 16 * q + i] = o[i];
-            else if (tid == SUR_ND)
+            if (t < SUR_ND)
+                store16(G + SUR_OFF_W1 + t * SUR_NH + 16 * q, o);
+            else if (t == SUR_ND)
                 for (int i = 0; i < 16; i++) G[SUR_OFF_B1 + 16 * q + i] = o[i];
         }
         // the tile's loss, in thread order
-        for (int o = 16; o > 0; o >>= 1) loss += __shfl_down_sync(0xffffffffu, loss, o);
-        if ((tid & 31) == 0) S.lsum[warp] = loss;
+        if (part == 0) {
+            for (int o = 16; o > 0; o >>= 1) loss += __shfl_down_sync(0xffffffffu, loss, o);
+            if ((tid & 31) == 0) S.lsum[warp] = loss;
+        }
         tc_fence_before();
         __syncthreads();  // TMEM reads and operand reads done before the next tile
         tc_fence_after();
@@ -393,7 +434,7 @@ cudaError_t launch_sur_grad_tc(const SurGradArgs& a, int sms, cudaStream_t st)
                                          (int)smem);
     if (e != cudaSuccess) return e;
     const long long grid = ntiles < (long long)sms ? ntiles : (long long)sms;
-    k_sur_grad_tc<<<(unsigned)grid, TR_M, smem, st>>>(a);
+    k_sur_grad_tc<<<(unsigned)grid, TR_T, smem, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -103,6 +103,9 @@ struct SurGradArgs {
     const float* T;           // [S][3] target forces
     const long long* idx;     // [batch] sample rows (nullptr: rows 0..batch-1)
     long long batch;
+    // tensor-core training: S > 0 draws the rows in the kernel (sur_sample)
+    unsigned long long seed;
+    long long step, S;
     const float* P;           // [SUR_NP] FP32 master parameters
     const float* mean;        // [32]
     const float* scale;       // [32]
@@ -114,6 +117,21 @@ struct SurGradArgs {
     const SurPacked* packed;
     int* status;
 };
+
+// minibatch row b of a step: splitmix64 output function (Steele, Lea & Flood
+// 2014) of a (seed, step, b) counter, modulo the S rows
+__device__ __forceinline__ unsigned long long mix64(unsigned long long z)
+{
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+__device__ __forceinline__ long long sur_sample(unsigned long long seed, long long step, long long b, long long S)
+{
+    unsigned long long z = mix64(seed + 0x9E3779B97F4A7C15ull * (unsigned long long)(step + 1));
+    z = mix64(z + 0x9E3779B97F4A7C15ull * (unsigned long long)(b + 1));
+    return (long long)(z % (unsigned long long)S);
+}
 
 constexpr int SUR_TILE = 64;      // samples per CTA of the training kernel
 constexpr int SUR_GRAD_THREADS = 256;
