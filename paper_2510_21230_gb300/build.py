@@ -16,7 +16,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libatm3.so")
 
-SOURCES = ["capi.cu", "atm_fwd.cu", "atm_list64.cu", "forces.cu", "md_kernels.cu", "atm_fp64.cu", "atm_fp32.cu", "atm_det64.cu",
+SOURCES = ["capi.cu", "atm_fwd.cu", "atm_list64.cu", "atm_prod.cu", "forces.cu", "md_kernels.cu", "atm_fp64.cu", "atm_fp32.cu", "atm_det64.cu",
            "atm_det32.cu", "noalloc.cu",
            "sur_kernels.cu", "sur_capi.cu", "sur_tc.cu", "sur_train_tc.cu", "peak.cu", "pair_masks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

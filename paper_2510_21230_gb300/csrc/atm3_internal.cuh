@@ -205,7 +205,61 @@ struct AtmArgs {
     // (ceil(16 edges / mcap)), so later launches can size the table from it
     // (nullptr: not recorded)
     int* emax;
+    // FP64 product rule: wrapped positions (original order, SoA [3n]) and the
+    // sorted -> original index
+    const double* x;
+    const int* perm;
 };
+
+constexpr int PROD_MAXW = 16;  // most warps of a product-rule CTA
+
+constexpr int PROD_COPIES = 8;  // of the FP32 forces
+
+// Shared memory of the product-rule kernel for a unit of M molecules: unit-frame
+// positions (FP32, FP64), sorted indices, the unit's sums (forces, or the FP64
+// pair scalars of 3c08 and 3c08a; 3c01 none)
+struct ProdSmem {
+    int off_frame, off_x, off_idx, off_acc, total;
+};
+// and per warp for molecules of up to n rows: the rows in pairs, again one by one,
+// the bounds of every eight, 3c08's anchor words, the queue, the bins, the staged
+// indices
+struct ProdWarpSmem {
+    int rows, eights, anch, queue, bins, rid, total;
+};
+
+template <typename R>
+__host__ __device__ inline ProdSmem prod_smem(int trav, int M)
+{
+    ProdSmem p;
+    long long o = 0;
+    auto al = [](long long v) { return (v + 15) & ~15ll; };
+    const bool f64 = sizeof(R) == 8;
+    p.off_frame = (int)o; o = al(o + 16ll * M);
+    p.off_x = (int)o;     o = al(o + (f64 ? 24ll * M : 0));
+    p.off_idx = (int)o;   o = al(o + 4ll * M);
+    p.off_acc = (int)o;
+    if (trav != 0) o = al(o + (f64 ? (trav != 1 ? 4ll * M * (M - 1) : 24ll * M) : 12ll * PROD_COPIES * M));
+    p.total = (int)(o < (1ll << 30) ? o : (1ll << 30));
+    return p;
+}
+
+template <typename R>
+__host__ __device__ inline ProdWarpSmem prod_warp_smem(int trav, int n)
+{
+    ProdWarpSmem p;
+    const bool f64 = sizeof(R) == 8;
+    const int rows = n < 32 ? 32 : (n + 31) & ~31;
+    int w = 16 * rows;
+    p.rows = w;    w += (f64 ? 32 : 16) * rows;
+    p.eights = w;  w += rows;
+    p.anch = w;    w += trav == 2 ? rows : 0;
+    p.queue = w;   w += f64 ? 256 : 0;
+    p.bins = w;    w += 128;
+    p.rid = w;     w += f64 ? 2 * rows : 0;
+    p.total = (w + 15) & ~15;
+    return p;
+}
 
 // Arguments of the forward-list kernel (atm_fwd.cuh: FP32C pair rule of 3c01,
 // 3c18 and 3c08).
@@ -534,6 +588,10 @@ cudaError_t launch_block_det64(int trav, int trunc, const AtmArgs<double>& a, in
                                size_t smem, int ctas, cudaStream_t s);
 cudaError_t launch_block_det32(int trav, int trunc, const AtmArgs<float>& a, int nwarps,
                                size_t smem, int ctas, cudaStream_t s);
+// the product-rule kernels of 3c18, 3c08 and the corner-anchored 3c08
+// (atm_prod.cu), one CTA of nwarps warps per unit
+template <typename R>
+cudaError_t launch_atm_prod(int trav, const AtmArgs<R>& a, int nwarps, cudaStream_t s);
 // the FP64 forward-list kernels (atm_list64.cu)
 cudaError_t launch_list64(const List64Args& a, cudaStream_t s);
 size_t list64_smem(int mcap, int run);

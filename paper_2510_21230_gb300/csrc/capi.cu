@@ -559,7 +559,9 @@ static bool fwd_active(const atm_ctx* c, int trav, int trunc, int prec)
     j.runs = c->d_runs;
     j.nruns = c->nruns;
     j.l64 = c->maxocc <= PM_CELL_MAX ? &c->l64 : nullptr;
-    return atm_uses_lists(j);
+    j.mcap = c->unit_max[trav];
+    j.x = c->x;
+    return atm_uses_lists(j) || atm_prod_plan(j).warps;
 }
 
 static void launch_choice(atm_ctx* c, int trav, int trunc, int prec, int mcap, int& persistent,
@@ -724,6 +726,8 @@ atm_status atm3::ctx_enqueue_forces(atm_ctx* c, int trav, int trunc, int prec, i
     j.lj_apart = prec != ATM_SURROGATE && !fused;
     j.runs = c->d_runs;
     j.nruns = c->nruns;
+    j.x = c->x;
+    j.perm = c->perm;
     if (!c->capturing) ctx_want_list64(c, trav, trunc, prec, j.mcap_fwd);
     j.l64 = c->maxocc <= PM_CELL_MAX ? &c->l64 : nullptr;
     const FwdLaunch fwd = atm_fwd_plan(j), l64 = atm_list64_plan(j);

@@ -81,6 +81,10 @@ struct ForceJob {
     // FP64 pair rule from forward lists (atm_list64.cu): the buffers and inputs
     // of List64Args (list nullptr: not taken), cells within PM_CELL_MAX
     const List64Args* l64 = nullptr;
+    // wrapped positions, original order, and the sorted -> original index (FP64
+    // product rule)
+    const double* x = nullptr;
+    const int* perm = nullptr;
     const int* runs = nullptr;  // FwdArgs.runs and nruns of FWD_RUN cells (device)
     long long nruns = 0;
 };
@@ -94,6 +98,12 @@ struct FwdLaunch {
 FwdLaunch atm_fwd_plan(const ForceJob& j);
 // the same for the FP64 lists (lj 1 or 2)
 FwdLaunch atm_list64_plan(const ForceJob& j);
+// the product-rule kernel's warps per CTA (0: the job does not take it) and bytes
+// of shared memory
+struct ProdLaunch {
+    int warps = 0, smem = 0;
+};
+ProdLaunch atm_prod_plan(const ForceJob& j);
 // either
 inline bool atm_uses_lists(const ForceJob& j)
 {

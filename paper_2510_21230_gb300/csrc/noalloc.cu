@@ -234,6 +234,8 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     j.unit_cnt2 = unit_cnt2;
     j.mcap_fwd = std::max(1, hocc[1 + ATM_FWD_UNIT]);
     j.whole = true;
+    j.x = x;
+    j.perm = perm;
     j.lj_apart = true;
     j.nruns = fwd_runs_of(rp.g);
     const FwdLaunch fwd = atm_fwd_plan(j);
