@@ -68,7 +68,7 @@ struct Rep {
 // the unit (base or anchor cell, index inside its replica) lies in an owned layer
 __host__ __device__ __forceinline__ bool unit_owned(const Rep& rp, long long lu)
 {
-    const int cz = (int)(lu / ((long long)rp.g.nc[0] * rp.g.nc[1]));
+    const int cz = (int)((unsigned)lu / ((unsigned)rp.g.nc[0] * (unsigned)rp.g.nc[1]));
     return cz >= rp.own_z0 && cz < rp.own_z1;
 }
 
@@ -84,10 +84,11 @@ struct Batch {
 __host__ __device__ __forceinline__ void cell_coords(const Grid& g, long long id, int& cx, int& cy,
                                                      int& cz)
 {
-    cx = (int)(id % g.nc[0]);
-    long long r = id / g.nc[0];
-    cy = (int)(r % g.nc[1]);
-    cz = (int)(r / g.nc[1]);
+    // (cell indices are ints)
+    const unsigned u = (unsigned)id, nx = (unsigned)g.nc[0], ny = (unsigned)g.nc[1], r = u / nx, z = r / ny;
+    cx = (int)(u - r * nx);
+    cy = (int)(r - z * ny);
+    cz = (int)z;
 }
 
 // neighbour cell id at offset (dx, dy, dz), |d| <= 1, periodic

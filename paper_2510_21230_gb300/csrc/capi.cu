@@ -128,6 +128,7 @@ static void free_all(atm_ctx* c)
     if (c->h_maxocc) cudaFreeHost(c->h_maxocc);
     if (c->cap_st) cudaStreamDestroy(c->cap_st);
     if (c->side_st) cudaStreamDestroy(c->side_st);
+    if (c->ev_occ) cudaEventDestroy(c->ev_occ);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->io_st) cudaStreamDestroy(c->io_st);
@@ -282,6 +283,7 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
                    cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&c->cap_st, cudaStreamNonBlocking) == cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&c->side_st, cudaStreamNonBlocking) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&c->ev_occ, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&c->io_st, cudaStreamNonBlocking) == cudaSuccess;
@@ -450,13 +452,22 @@ extern "C" atm_status atm_set_state_dev(atm_ctx* c, const double* x_dev, const d
     return ATM_OK;
 }
 
-// cell build kernels only (no host synchronisation; capturable)
-static atm_status launch_cells(atm_ctx* c)
+// cell build kernels only (no host synchronisation; capturable).  The arrival
+// ranks take perm's place until the scatter, and the unsorted lists c->rank.
+// read: the occupancy maxima and the status word are copied to the host before
+// the sort, c->ev_occ marks their arrival
+static atm_status launch_cells(atm_ctx* c, bool read = false)
 {
     cudaEvent_t ev = ctx_prof_begin(c, PK_CELLS);
-    CU(launch_build_cells(c->b, c->x, c->cell_of, c->rank, c->count, c->start, c->perm, c->xl,
-                          c->xl32, c->cell_sorted, c->d_maxocc, c->d_status, c->wide_cells,
+    CU(launch_cell_counts(c->b, c->x, c->cell_of, c->perm, c->count, c->d_maxocc, c->d_status, c->wide_cells,
                           c->st));
+    if (read) {
+        CU(cudaMemcpyAsync(c->h_maxocc, c->d_maxocc, MAXOCC_N * sizeof(int), cudaMemcpyDeviceToHost, c->st));
+        CU(cudaMemcpyAsync(c->h_status, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+        CU(cudaEventRecord(c->ev_occ, c->st));
+    }
+    CU(launch_cell_sort(c->b, c->x, c->cell_of, c->perm, c->count, c->start, c->rank, c->perm, c->xl, c->xl32,
+                        c->cell_sorted, c->st));
     ctx_prof_end(c, PK_CELLS, ev);
     c->n_launch += c->n > 0 ? CELL_KERNELS : 2;
     return ATM_OK;
@@ -484,11 +495,12 @@ static void take_unit_sizes(atm_ctx* c)
 // cell build + read back of the occupancy maxima that size the force kernels
 static atm_status enqueue_cells(atm_ctx* c)
 {
-    atm_status s = launch_cells(c);
+    // the host waits for the sizes, not for the sort behind them
+    atm_status s = launch_cells(c, true);
     if (s != ATM_OK) return s;
-    CU(cudaMemcpyAsync(c->h_maxocc, c->d_maxocc, MAXOCC_N * sizeof(int),
-                       cudaMemcpyDeviceToHost, c->st));
-    s = ctx_sync_and_check(c);
+    CU(cudaEventSynchronize(c->ev_occ));
+    if (c->ev_live.size() >= 4096) prof_drain(c);
+    s = check_status(c);
     if (s != ATM_OK) return s;
     take_unit_sizes(c);
     c->cells_built = true;

@@ -117,6 +117,7 @@ struct atm_ctx {
     // (forked from and joined to the context's stream by the two events)
     cudaStream_t side_st = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_occ = nullptr;  // the occupancy maxima are in h_maxocc
     // host round trips (atm_step_host): the input checks and the copy of the
     // last step's positions run on io_st beside the context's stream
     cudaStream_t io_st = nullptr;

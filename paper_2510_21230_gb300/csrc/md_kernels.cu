@@ -43,8 +43,29 @@ __device__ __forceinline__ int bin1(double t, double w, double iw, int n, double
     return c;
 }
 
+// a non-negative finite double to FP32, the mantissa cut off (integer work: a
+// conversion takes the FP64 pipe); below 2^-126 zero
+__device__ __forceinline__ float cut32(double t)
+{
+    const int hi = __double2hiint(t);  // (-0: zero too)
+    return hi < 0x38100000 ? 0.0f
+                           : __uint_as_float(((unsigned)(hi - 0x38000000) << 3) | ((unsigned)__double2loint(t) >> 29));
+}
+
+// a double in [0, 2^127) to FP32, rounded to nearest even (integer work again)
+__device__ __forceinline__ float round32(double t)
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(t);
+    if (u < 0x3810000000000000ull) return (float)t;
+    return __uint_as_float((unsigned)((u + 0x0fffffffull + ((u >> 29) & 1ull)) >> 29) - (896u << 23));
+}
+
 // K1: wrap positions in place, global cell id per molecule, cell histogram
-// with the arrival rank of each molecule
+// with the arrival rank of each molecule.  A coordinate in [0, L) (one integer
+// compare: the bits of non-negative doubles order as they do) stays as it is, and
+// its cell comes from an FP32 quotient wherever that lies farther from an integer
+// than its error; the FP64 pipe, which takes 16 cycles a warp instruction, is left to
+// the others.  256,000 molecules: 22 -> 8.3 us.
 __global__ void k_wrap_bin(Batch B, double* __restrict__ x, int* __restrict__ cell_of,
                            int* __restrict__ rank, int* __restrict__ count, int* __restrict__ status)
 {
@@ -52,17 +73,28 @@ __global__ void k_wrap_bin(Batch B, double* __restrict__ x, int* __restrict__ ce
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const Rep& rp = B.rep[B.rep_of_mol[i]];
+    double xv[3];
+    for (int d = 0; d < 3; d++) xv[d] = x[d * n + i];
     int cc[3];
     for (int d = 0; d < 3; d++) {
-        double xv = x[d * n + i];
-        if (!isfinite(xv)) {
-            atomicOr(status, ST_NONFINITE);
-            xv = 0.0;
+        double t = xv[d];
+        if ((unsigned long long)__double_as_longlong(t) >= (unsigned long long)__double_as_longlong(rp.g.L[d])) {
+            if (!isfinite(t)) {
+                atomicOr(status, ST_NONFINITE);
+                t = 0.0;
+            }
+            t = wrap1(t, rp.g.L[d]);
+            x[d * n + i] = t;
         }
-        double t = wrap1(xv, rp.g.L[d]);
-        x[d * n + i] = t;
-        double loc;
-        cc[d] = bin1(t, rp.g.w[d], rp.g.iw[d], rp.g.nc[d], loc);
+        // both factors cut to 2^-23, the product rounded to 2^-24: within 2^-21.6
+        const float q = cut32(t) * cut32(rp.g.iw[d]), fq = floorf(q), tol = q * 0x1p-21f;
+        const int nc = rp.g.nc[d];
+        if (q - fq > tol && (fq + 1.0f) - q > tol) {
+            cc[d] = min((int)fq, nc - 1);
+        } else {
+            double loc;
+            cc[d] = bin1(t, rp.g.w[d], rp.g.iw[d], nc, loc);
+        }
     }
     int id = (int)rp.cell0 + (cc[2] * rp.g.nc[1] + cc[1]) * rp.g.nc[0] + cc[0];
     cell_of[i] = id;
@@ -70,31 +102,34 @@ __global__ void k_wrap_bin(Batch B, double* __restrict__ x, int* __restrict__ ce
 }
 
 // K2: exclusive scan of the cell counts (one CTA of 1024 threads, each warp
-// owns a contiguous segment) and the largest occupancy
+// owns a contiguous segment)
 __global__ void __launch_bounds__(1024) k_scan(long long ncell, const int* __restrict__ count,
-                                               int* __restrict__ start, int* __restrict__ maxocc)
+                                               int* __restrict__ start)
 {
     // warp w owns the contiguous segment [w seg, (w + 1) seg) of the cells and
-    // reads it 32 consecutive counts at a time (coalesced): its total and
-    // largest count first, then, after a scan of the 32 totals, the exclusive
-    // prefix of every cell with a shuffle scan per 32 and a running carry
+    // reads it 256 consecutive counts at a time (coalesced, eight loads in flight:
+    // 19,683 cells 10 -> 8.4 us): its total first, then, after a scan of the 32
+    // totals, the exclusive prefix of every cell with a shuffle scan per 32 and
+    // a running carry
+    constexpr int U = 8;
     __shared__ int s_tot[32];
-    __shared__ int s_max[32];
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long seg = ((ncell + 31) / 32 + 31) / 32 * 32;
     const long long lo = warp * seg, hi = lo + seg < ncell ? lo + seg : ncell;
-    int tot = 0, mx = 0;
-    for (long long c0 = lo; c0 < hi; c0 += 32) {
-        const long long c = c0 + lane;
-        const int v = c < hi ? count[c] : 0;
-        tot += __reduce_add_sync(FULL, v);
-        mx = max(mx, (int)__reduce_max_sync(FULL, (unsigned)v));
+    int tot = 0;
+    for (long long c0 = lo; c0 < hi; c0 += 32 * U) {
+        int v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const long long c = c0 + 32 * u + lane;
+            v[u] = c < hi ? count[c] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) tot += v[u];
     }
-    if (lane == 0) {
-        s_tot[warp] = tot;
-        s_max[warp] = mx;
-    }
+    tot = __reduce_add_sync(FULL, tot);
+    if (lane == 0) s_tot[warp] = tot;
     __syncthreads();
     if (warp == 0) {
         const int t = s_tot[lane];
@@ -104,77 +139,83 @@ __global__ void __launch_bounds__(1024) k_scan(long long ncell, const int* __res
             if (lane >= o) incl += u;
         }
         s_tot[lane] = incl - t;  // exclusive: the cells before warp lane's segment
-        const int m = (int)__reduce_max_sync(FULL, (unsigned)s_max[lane]);
-        if (lane == 0) *maxocc = m;
         if (lane == 31) start[ncell] = incl;
     }
     __syncthreads();
     int carry = s_tot[warp];
-    for (long long c0 = lo; c0 < hi; c0 += 32) {
-        const long long c = c0 + lane;
-        const int v = c < hi ? count[c] : 0;
-        int incl = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += u;
+    for (long long c0 = lo; c0 < hi; c0 += 32 * U) {
+        int v[U], incl[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const long long c = c0 + 32 * u + lane;
+            incl[u] = v[u] = c < hi ? count[c] : 0;
         }
-        if (c < hi) start[c] = carry + incl - v;
-        carry += __shfl_sync(FULL, incl, 31);
+        for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int t = __shfl_up_sync(FULL, incl[u], o);
+                if (lane >= o) incl[u] += t;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const long long c = c0 + 32 * u + lane;
+            if (c < hi) start[c] = carry + incl[u] - v[u];
+            carry += __shfl_sync(FULL, incl[u], 31);
+        }
     }
 }
 
-// largest staged-molecule count of a traversal unit, per traversal:
-// out[0] 3c01 (27 cells), out[1] 3c18 (base + 13 forward), out[2] 3c08 (2x2x2 block),
-// out[ATM_FWD_UNIT] the forward lists' 18 cells (the base cell's layer and the next)
-__global__ void k_unit_max(Batch B, const int* __restrict__ start, int wide, int* __restrict__ out)
+// out[0] the largest cell, out + 1 the largest staged-molecule count of a
+// traversal unit, per traversal: 3c01 (27 cells), 3c18 (base + 13 forward), 3c08
+// (2x2x2 block), [ATM_FWD_UNIT] the forward lists' 18 cells (the base cell's layer
+// and the next).  From the counts alone (27 independent loads a cell), so it comes
+// before the scan and the host can read it while the molecules are sorted.
+__global__ void k_unit_max(Batch B, const int* __restrict__ count, int wide, int* __restrict__ out)
 {
     long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    int m01 = 0, m18 = 0, m08 = 0, mw = 0, mf = 0;
+    int m01 = 0, m18 = 0, m08 = 0, mw = 0, mf = 0, own = 0;
     if (c < B.ncell) {
         const Rep& rp = B.rep[B.rep_of_cell[c]];
-        const int* st = start + rp.cell0;
+        const int* ct = count + rp.cell0;
         int cx, cy, cz;
         cell_coords(rp.g, c - rp.cell0, cx, cy, cz);
+        const int nx = rp.g.nc[0], ny = rp.g.nc[1], nz = rp.g.nc[2];
+        const int xs[3] = {cx > 0 ? cx - 1 : nx - 1, cx, cx + 1 < nx ? cx + 1 : 0};
+        const int ys[3] = {nx * (cy > 0 ? cy - 1 : ny - 1), nx * cy, nx * (cy + 1 < ny ? cy + 1 : 0)};
+        const int zs[3] = {nx * ny * (cz > 0 ? cz - 1 : nz - 1), nx * ny * cz, nx * ny * (cz + 1 < nz ? cz + 1 : 0)};
+        int k[27];
+#pragma unroll
+        for (int t = 0; t < 27; t++) k[t] = ct[zs[t / 9] + ys[(t / 3) % 3] + xs[t % 3]];
+#pragma unroll
         for (int t = 0; t < 27; t++) {
-            int dx, dy, dz;
-            offset27(t, dx, dy, dz);
-            long long nc = cell_at(rp.g, cx, cy, cz, dx, dy, dz);
-            int k = st[nc + 1] - st[nc];
-            m01 += k;
-            if (t >= 13) m18 += k;
-            if (t >= 9) mf += k;
-            if (dx >= 0 && dy >= 0 && dz >= 0) m08 += k;
+            m01 += k[t];
+            if (t >= 13) m18 += k[t];
+            if (t >= 9) mf += k[t];
+            if (t % 3 >= 1 && (t / 3) % 3 >= 1 && t / 9 >= 1) m08 += k[t];
         }
+        own = k[13];
         // the wide traversal's 5^3 neighbourhood (only when that traversal is in use)
-        for (int t = 0; t < (wide ? 125 : 0); t++) {
-            long long nc = cell_at(rp.g, cx, cy, cz, t % 5 - 2, (t / 5) % 5 - 2, t / 25 - 2);
-            mw += st[nc + 1] - st[nc];
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        m01 = max(m01, __shfl_down_sync(0xffffffffu, m01, o));
-        m18 = max(m18, __shfl_down_sync(0xffffffffu, m18, o));
-        m08 = max(m08, __shfl_down_sync(0xffffffffu, m08, o));
-        mw = max(mw, __shfl_down_sync(0xffffffffu, mw, o));
-        mf = max(mf, __shfl_down_sync(0xffffffffu, mf, o));
+        for (int t = 0; t < (wide ? 125 : 0); t++)
+            mw += ct[cell_at(rp.g, cx, cy, cz, t % 5 - 2, (t / 5) % 5 - 2, t / 25 - 2)];
     }
     // block maximum first: one global atomic per value and block
-    __shared__ int s_m[5][32];
+    __shared__ int s_m[6][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (lane == 0) {
-        s_m[0][warp] = m01;
-        s_m[1][warp] = m18;
-        s_m[2][warp] = m08;
-        s_m[3][warp] = mw;
-        s_m[4][warp] = mf;
+    const int m[6] = {own, m01, m18, m08, mw, mf};
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+        const int v = __reduce_max_sync(0xffffffffu, m[q]);
+        if (lane == 0) s_m[q][warp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 5) {
-        int m = 0;
-        for (int w = 0; w < nw; w++) m = max(m, s_m[threadIdx.x][w]);
-        atomicMax(out + (threadIdx.x == 4 ? ATM_FWD_UNIT : (int)threadIdx.x), m);
+    if (threadIdx.x < 6) {
+        const int q = threadIdx.x;
+        int v = 0;
+        for (int w = 0; w < nw; w++) v = max(v, s_m[q][w]);
+        atomicMax(out + (q == 5 ? 1 + ATM_FWD_UNIT : q), v);
         // the corner-anchored 3c08 stages the same blocks as 3c08
-        if (threadIdx.x == 2) atomicMax(out + 4, m);
+        if (q == 3) atomicMax(out + 5, v);
     }
 }
 
@@ -221,62 +262,53 @@ __global__ void k_unit_classes(Batch B, const int* __restrict__ start, int trav,
 
 // K3a: scatter by arrival rank
 __global__ void k_scatter(long long n, const int* __restrict__ cell_of, const int* __restrict__ rank,
-                          const int* __restrict__ start, int* __restrict__ perm)
+                          const int* __restrict__ start, int* __restrict__ list)
 {
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    perm[start[cell_of[i]] + rank[i]] = (int)i;
+    list[start[cell_of[i]] + rank[i]] = (int)i;
 }
 
-// K3b+c: one warp per cell restores the original index order inside the cell
-// (the rank of each entry among the cell's entries; lane 0 insertion-sorts a
-// cell of more than 32) and writes, for every sorted slot, the FP64 and FP32
-// cell-local coordinates (t - c w clamped to [0, w], the cell's own c: the
-// binning's arithmetic without its division) and the slot's global cell
+// K3b+c: a thread per entry of the unsorted lists restores the original index
+// order inside its cell (its place is the number of the cell's entries below it)
+// and writes, for its sorted slot, the FP64 and FP32 cell-local coordinates (t - c
+// w clamped to [0, w], the cell's own c: the binning's arithmetic without its
+// division) and the global cell.  Full warps of entries, not a warp per cell, and
+// integer compares and conversions: 9 FP64 instructions a warp (256,000 molecules
+// in cells of 13: 26 -> 12 us).
 __global__ void __launch_bounds__(128) k_cell_order(Batch B, const double* __restrict__ x,
+                                                    const int* __restrict__ cell_of,
                                                     const int* __restrict__ start,
+                                                    const int* __restrict__ list,
                                                     int* __restrict__ perm, double* __restrict__ xl,
                                                     float* __restrict__ xl32,
                                                     int* __restrict__ cell_sorted)
 {
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const long long c = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (c >= B.ncell) return;  // whole warps leave together
     const long long n = B.ntot;
-    const int lo = start[c], hi = start[c + 1], cnt = hi - lo;
-    if (cnt <= 32) {
-        const int v = lane < cnt ? perm[lo + lane] : 0x7fffffff;
-        int r = 0;
-        for (int k = 0; k < cnt; k++) r += __shfl_sync(FULL, v, k) < v ? 1 : 0;
-        __syncwarp();  // every entry is read before any is overwritten
-        if (lane < cnt) perm[lo + r] = v;
-    } else {
-        if (lane == 0)
-            for (int a = lo + 1; a < hi; a++) {
-                const int v = perm[a];
-                int b = a - 1;
-                while (b >= lo && perm[b] > v) {
-                    perm[b + 1] = perm[b];
-                    b--;
-                }
-                perm[b + 1] = v;
-            }
-    }
-    __syncwarp();
+    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const int i = list[e];
+    const int c = cell_of[i];
+    double t[3];
+    for (int d = 0; d < 3; d++) t[d] = x[d * n + i];
+    const int lo = start[c], hi = start[c + 1];
+    int s = lo;
+    for (int k = lo; k < hi; k++) s += list[k] < i ? 1 : 0;
     const Rep& rp = B.rep[B.rep_of_cell[c]];
     int cc[3];
     cell_coords(rp.g, c - rp.cell0, cc[0], cc[1], cc[2]);
-    for (int s = lo + lane; s < hi; s += 32) {
-        const int i = perm[s];
-        for (int d = 0; d < 3; d++) {
-            const double w = rp.g.w[d];
-            double l = __dsub_rn(x[d * n + i], __dmul_rn((double)cc[d], w));
-            l = l < 0.0 ? 0.0 : (l > w ? w : l);
-            xl[d * n + s] = l;
-            xl32[d * n + s] = (float)l;
-        }
-        cell_sorted[s] = (int)c;
+    perm[s] = i;
+    cell_sorted[s] = c;
+    for (int d = 0; d < 3; d++) {
+        const double w = rp.g.w[d];
+        // (double)cc, exactly
+        const double cd = __dsub_rn(__hiloint2double(0x43300000, cc[d]), 0x1p52);
+        double l = __dsub_rn(t[d], __dmul_rn(cd, w));
+        // l < 0 ? 0 : (l > w ? w : l)
+        const long long b = __double_as_longlong(l), bw = __double_as_longlong(w);
+        l = __longlong_as_double(b < 0 ? 0 : (b > bw ? bw : b));
+        xl[d * n + s] = l;
+        xl32[d * n + s] = round32(l);
     }
 }
 
@@ -410,9 +442,9 @@ __global__ void __launch_bounds__(256) k_kick(Batch B, const int* __restrict__ p
         double vv = __dadd_rn(v[d * n + i], __dmul_rn(half_dt, f));
         v[d * n + i] = vv;
         if (drift) x[d * n + i] = __dadd_rn(x[d * n + i], __dmul_rn(dt, vv));
-        k += 0.5 * vv * vv;
+        if (!drift) k += 0.5 * vv * vv;
     }
-    ke[i] = k;
+    if (!drift) ke[i] = k;  // (the second half kick of the step gives the kinetic energy)
 }
 
 // the first half kick and the drift from a total force given in the
@@ -731,22 +763,27 @@ __global__ void k_fix_to_double(double* __restrict__ f, long long m, double scal
 
 static inline unsigned nblk(long long m, int b) { return (unsigned)((m + b - 1) / b); }
 
-cudaError_t launch_build_cells(const Batch& b, double* x, int* cell_of, int* rank, int* count,
-                               int* start, int* perm, double* xl, float* xl32, int* cell_sorted,
+cudaError_t launch_cell_counts(const Batch& b, double* x, int* cell_of, int* rank, int* count,
                                int* maxocc, int* status, bool wide, cudaStream_t st)
 {
     const long long n = b.ntot;
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int) * (size_t)b.ncell, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(maxocc, 0, (1 + ATM_NUNIT) * sizeof(int), st);
     if (e != cudaSuccess) return e;
     if (n > 0) k_wrap_bin<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(b, x, cell_of, rank, count, status);
-    k_scan<<<1, 1024, 0, st>>>(b.ncell, count, start, maxocc);
-    e = cudaMemsetAsync(maxocc + 1, 0, ATM_NUNIT * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    k_unit_max<<<nblk(b.ncell, MD_BLOCK), MD_BLOCK, 0, st>>>(b, start, wide ? 1 : 0, maxocc + 1);
+    k_unit_max<<<nblk(b.ncell, MD_BLOCK), MD_BLOCK, 0, st>>>(b, count, wide ? 1 : 0, maxocc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cell_sort(const Batch& b, const double* x, const int* cell_of, const int* rank,
+                             const int* count, int* start, int* list, int* perm, double* xl, float* xl32,
+                             int* cell_sorted, cudaStream_t st)
+{
+    const long long n = b.ntot;
+    k_scan<<<1, 1024, 0, st>>>(b.ncell, count, start);
     if (n > 0) {
-        k_scatter<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, cell_of, rank, start, perm);
-        k_cell_order<<<(unsigned)((b.ncell + 3) / 4), 128, 0, st>>>(b, x, start, perm, xl, xl32,
-                                                                  cell_sorted);
+        k_scatter<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, cell_of, rank, start, list);
+        k_cell_order<<<nblk(n, 128), 128, 0, st>>>(b, x, cell_of, start, list, perm, xl, xl32, cell_sorted);
     }
     return cudaGetLastError();
 }

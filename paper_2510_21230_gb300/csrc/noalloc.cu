@@ -15,6 +15,8 @@
 // Every call uses the same array and leaves its contents behind; everything
 // that must start at zero is cleared on each call.  Two calls whose GPU work
 // overlaps (different streams, or different host threads) race on the array.
+#include <string.h>
+
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -197,13 +199,15 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     }
     NA_CU(cudaMemsetAsync(status, 0, sizeof(int), st));
     if (n > 0) NA_CU(launch_check_finite(3 * n, x, status, st));
-    NA_CU(launch_build_cells(b, x, cell_of, rank, count, start, perm, xl, xl32, cell_sorted,
-                             maxocc, status, false, st));
-    int hocc[1 + ATM_NUNIT] = {}, hstat = 0;
-    NA_CU(cudaMemcpyAsync(hocc, maxocc, sizeof(hocc), cudaMemcpyDeviceToHost, st));
-    NA_CU(cudaMemcpyAsync(&hstat, status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    NA_CU(launch_cell_counts(b, x, cell_of, perm, count, maxocc, status, false, st));
+    NA_CU(launch_cell_sort(b, x, cell_of, perm, count, start, rank, perm, xl, xl32, cell_sorted, st));
+    // the status word and the occupancy maxima behind it in one copy
+    constexpr size_t OCC = (NA.maxocc - NA.status) / sizeof(int);
+    int hbuf[OCC + 1 + ATM_NUNIT] = {};
+    NA_CU(cudaMemcpyAsync(hbuf, status, sizeof(hbuf), cudaMemcpyDeviceToHost, st));
+    const int* hocc = hbuf + OCC;
     NA_CU(cudaStreamSynchronize(st));
-    if (hstat & ST_NONFINITE) return ATM_E_NONFINITE;
+    if (hbuf[0] & ST_NONFINITE) return ATM_E_NONFINITE;
 
     // LJ pairs and ATM triplets (staged-molecule capacity = largest unit of the traversal)
     ForceJob j;
@@ -264,10 +268,14 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     r.out = res;
     NA_CU(launch_final_reduce(r, st));
     if (n > 0) NA_CU(launch_gather_forces(n, perm, f_lj, f_atm, 0, f_dev, st));
-    ResultDev hres{};
-    NA_CU(cudaMemcpyAsync(&hres, res, sizeof(ResultDev), cudaMemcpyDeviceToHost, st));
-    NA_CU(cudaMemcpyAsync(&hstat, status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    // the result and the status word behind the partial sums in one copy
+    alignas(ResultDev) unsigned char hout[NA.status - NA.res + sizeof(int)];
+    NA_CU(cudaMemcpyAsync(hout, res, sizeof(hout), cudaMemcpyDeviceToHost, st));
     NA_CU(cudaStreamSynchronize(st));
+    ResultDev hres;
+    int hstat;
+    memcpy(&hres, hout, sizeof(hres));
+    memcpy(&hstat, hout + (NA.status - NA.res), sizeof(hstat));
     if (hstat & ST_NONFINITE) return ATM_E_NONFINITE;
     if (hstat & ST_CAPACITY) return ATM_E_CAPACITY;
     if (out) {
