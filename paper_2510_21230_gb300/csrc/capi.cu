@@ -1475,7 +1475,7 @@ extern "C" atm_status atm_rdf_accumulate(atm_ctx* c, double r_max, int nbins)
     if (c->rdf_samples > 0 && (r_max != c->rdf_rmax || nbins != c->rdf_nbins))
         return ctx_fail(c, ATM_E_STATE, "the RDF accumulator holds another range/bin count; reset it");
     CU(cudaSetDevice(c->device));
-    CU(launch_rdf(c->b, c->xl, c->start, c->cell_sorted, r_max, nbins, c->d_rdf, c->st));
+    CU(launch_rdf(c->b, c->xl, c->xl32, c->start, c->cell_sorted, r_max, nbins, c->d_rdf, c->st));
     c->n_launch += 1;
     c->rdf_rmax = r_max;
     c->rdf_nbins = nbins;

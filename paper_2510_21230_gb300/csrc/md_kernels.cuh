@@ -91,8 +91,8 @@ cudaError_t launch_gather_forces(long long n, const int* perm, const double* f_l
 // adds the pair-distance histogram (nbins equal bins over [0, rmax), every
 // pair once, rmax at most the smallest cell edge) of every replica to
 // counts[R * nbins]
-cudaError_t launch_rdf(const Batch& b, const double* xl, const int* start, const int* cell_sorted,
-                       double rmax, int nbins, unsigned long long* counts, cudaStream_t st);
+cudaError_t launch_rdf(const Batch& b, const double* xl, const float* xl32, const int* start,
+                       const int* cell_sorted, double rmax, int nbins, unsigned long long* counts, cudaStream_t st);
 // adds the histogram of coordinate `axis` (nbins equal bins over [0, L_axis))
 // of every replica's wrapped positions to counts[R * nbins]
 cudaError_t launch_density(const Batch& b, const double* x, int axis, int nbins,
