@@ -115,15 +115,14 @@ static void free_all(atm_ctx* c)
     sur_free(c);
     void* dev[] = {c->d_rep, c->d_rep_of_cell, c->d_rep_of_mol, c->x, c->v, c->x0, c->v0, c->xl,
                    c->xl32, c->cell_of, c->rank, c->count, c->start, c->perm, c->cell_sorted,
-                   c->f_lj, c->f_atm, c->f_out, c->unit_ew, c->unit_cnt, c->mol_ew, c->mol_cnt,
-                   c->ke, c->d_res, c->d_part, c->d_status, c->d_maxocc, c->d_work, c->d_dens,
+                   c->f_lj, c->f_out, c->unit_ew, c->unit_cnt, c->mol_ew, c->mol_cnt,
+                   c->ke, c->d_res, c->d_part, c->d_maxocc, c->d_work, c->d_dens,
                    c->d_rdf, c->d_ttarget, c->unit_ew2, c->unit_cnt2, c->f_in, c->d_chk,
                    c->d_ulist, c->d_ucount, c->d_runs, c->pmask, c->l64.list, c->l64.G, c->l64.place,
                    c->l64.count, c->l64.mol_w3, c->l64.mol_n3};
     for (void* p : dev)
         if (p) cudaFree(p);
     if (c->h_res) cudaFreeHost(c->h_res);
-    if (c->h_status) cudaFreeHost(c->h_status);
     if (c->h_chk) cudaFreeHost(c->h_chk);
     if (c->h_maxocc) cudaFreeHost(c->h_maxocc);
     if (c->cap_st) cudaStreamDestroy(c->cap_st);
@@ -245,8 +244,8 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
     ok = ok && alloc((void**)&c->start, (NC + 1) * sizeof(int));
     ok = ok && alloc((void**)&c->perm, N * sizeof(int));
     ok = ok && alloc((void**)&c->cell_sorted, N * sizeof(int));
-    ok = ok && alloc((void**)&c->f_lj, 3 * N * sizeof(double));
-    ok = ok && alloc((void**)&c->f_atm, 3 * N * sizeof(double));
+    ok = ok && alloc((void**)&c->f_lj, 6 * N * sizeof(double));
+    c->f_atm = c->f_lj + 3 * N;  // (zeroed together)
     ok = ok && alloc((void**)&c->f_out, 3 * N * sizeof(double));
     ok = ok && alloc((void**)&c->f_in, 3 * N * sizeof(double));
     ok = ok && alloc((void**)&c->d_chk, sizeof(int));
@@ -260,10 +259,11 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
     ok = ok && alloc((void**)&c->ke, N * sizeof(double));
     ok = ok && alloc((void**)&c->d_res, nrep * sizeof(ResultDev));
     ok = ok && alloc((void**)&c->d_part, (size_t)nrep * REDUCE_PARTS * sizeof(ResultDev));
-    ok = ok && alloc((void**)&c->d_status, sizeof(int));
-    // largest cell, largest unit per traversal, edge-table need per traversal
-    ok = ok && alloc((void**)&c->d_maxocc, MAXOCC_N * sizeof(int));
-    ok = ok && cudaMemset(c->d_maxocc, 0, MAXOCC_N * sizeof(int)) == cudaSuccess;
+    // largest cell, largest unit per traversal, edge-table need per traversal; the
+    // status word (read back together)
+    ok = ok && alloc((void**)&c->d_maxocc, (MAXOCC_N + 1) * sizeof(int));
+    ok = ok && cudaMemset(c->d_maxocc, 0, (MAXOCC_N + 1) * sizeof(int)) == cudaSuccess;
+    c->d_status = c->d_maxocc + MAXOCC_N;
     ok = ok && alloc((void**)&c->d_work, 4 * sizeof(int));
     ok = ok && alloc((void**)&c->d_ulist, 3 * NC * sizeof(int));
     ok = ok && alloc((void**)&c->d_ucount, 4 * sizeof(int));
@@ -274,9 +274,9 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
     ok = ok && alloc((void**)&c->d_ttarget, nrep * sizeof(double));
     ok = ok && alloc((void**)&c->pmask, atm3::PM_WORDS * N * sizeof(unsigned));
     ok = ok && cudaMallocHost((void**)&c->h_res, nrep * sizeof(ResultDev)) == cudaSuccess;
-    ok = ok && cudaMallocHost((void**)&c->h_status, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&c->h_chk, sizeof(int)) == cudaSuccess;
-    ok = ok && cudaMallocHost((void**)&c->h_maxocc, MAXOCC_N * sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMallocHost((void**)&c->h_maxocc, (MAXOCC_N + 1) * sizeof(int)) == cudaSuccess;
+    c->h_status = c->h_maxocc + MAXOCC_N;
     ok = ok && cudaDeviceGetAttribute(&c->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin,
                                       c->device) == cudaSuccess;
     ok = ok && cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) ==
@@ -312,7 +312,8 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
         ok = ok && cudaMemcpy(c->d_rep_of_mol, rom.data(), N * sizeof(int),
                               cudaMemcpyHostToDevice) == cudaSuccess;
     }
-    ok = ok && cudaMemsetAsync(c->d_status, 0, sizeof(int), c->st) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(c->d_maxocc, 0, (MAXOCC_N + 1) * sizeof(int), c->st) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(c->count, 0, NC * sizeof(int), c->st) == cudaSuccess;
     ok = ok && cudaMemsetAsync(c->v, 0, 3 * N * sizeof(double), c->st) == cudaSuccess;
     ok = ok && cudaMemsetAsync(c->mol_ew, 0, 2 * N * sizeof(double), c->st) == cudaSuccess;
     ok = ok && cudaMemsetAsync(c->mol_cnt, 0, 2 * N * sizeof(unsigned), c->st) == cudaSuccess;
@@ -439,13 +440,15 @@ extern "C" atm_status atm_set_state_dev(atm_ctx* c, const double* x_dev, const d
     size_t bytes = 3 * (size_t)c->n * sizeof(double);
     if (bytes) {
         CU(cudaMemcpyAsync(c->x, x_dev, bytes, cudaMemcpyDeviceToDevice, c->st));
-        if (v_dev)
-            CU(cudaMemcpyAsync(c->v, v_dev, bytes, cudaMemcpyDeviceToDevice, c->st));
-        else
-            CU(cudaMemsetAsync(c->v, 0, bytes, c->st));
         CU(launch_check_finite(3 * c->n, c->x, c->d_status, c->st));
-        CU(launch_check_finite(3 * c->n, c->v, c->d_status, c->st));
-        c->n_launch += 2;
+        c->n_launch += 1;
+        if (v_dev) {
+            CU(cudaMemcpyAsync(c->v, v_dev, bytes, cudaMemcpyDeviceToDevice, c->st));
+            CU(launch_check_finite(3 * c->n, c->v, c->d_status, c->st));
+            c->n_launch += 1;
+        } else {
+            CU(cudaMemsetAsync(c->v, 0, bytes, c->st));
+        }
     }
     c->have_x = true;
     invalidate(c);
@@ -462,8 +465,7 @@ static atm_status launch_cells(atm_ctx* c, bool read = false)
     CU(launch_cell_counts(c->b, c->x, c->cell_of, c->perm, c->count, c->d_maxocc, c->d_status, c->wide_cells,
                           c->st));
     if (read) {
-        CU(cudaMemcpyAsync(c->h_maxocc, c->d_maxocc, MAXOCC_N * sizeof(int), cudaMemcpyDeviceToHost, c->st));
-        CU(cudaMemcpyAsync(c->h_status, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+        CU(cudaMemcpyAsync(c->h_maxocc, c->d_maxocc, (MAXOCC_N + 1) * sizeof(int), cudaMemcpyDeviceToHost, c->st));
         CU(cudaEventRecord(c->ev_occ, c->st));
     }
     CU(launch_cell_sort(c->b, c->x, c->cell_of, c->perm, c->count, c->start, c->rank, c->perm, c->xl, c->xl32,

@@ -341,6 +341,15 @@ cudaError_t enqueue_atm(const ForceJob& j, size_t* smem_set, bool* capacity)
     return e;
 }
 
+// f_atm, and f_lj too, to zero (one operation where f_atm follows f_lj)
+static cudaError_t zero_forces(const ForceJob& j, bool lj)
+{
+    const size_t m = 3 * (size_t)j.b.ntot;
+    if (lj && j.f_atm == j.f_lj + m) return cudaMemsetAsync(j.f_lj, 0, 2 * m * sizeof(double), j.st);
+    const cudaError_t e = cudaMemsetAsync(j.f_atm, 0, m * sizeof(double), j.st);
+    return e == cudaSuccess && lj ? cudaMemsetAsync(j.f_lj, 0, m * sizeof(double), j.st) : e;
+}
+
 static cudaError_t enqueue_atm_launches(const ForceJob& j, size_t* smem_set, bool* capacity)
 {
     *capacity = false;
@@ -356,14 +365,12 @@ static cudaError_t enqueue_atm_launches(const ForceJob& j, size_t* smem_set, boo
     cudaError_t e;
     const FwdLaunch f = atm_fwd_plan(j), f64 = atm_list64_plan(j);
     if (f64.use && j.b.ntot > 0) {
-        e = cudaMemsetAsync(j.f_atm, 0, 3 * (size_t)j.b.ntot * sizeof(double), j.st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(j.f_lj, 0, 3 * (size_t)j.b.ntot * sizeof(double), j.st);
+        e = zero_forces(j, true);
         return e == cudaSuccess ? launch_l64(j, f64) : e;
     }
     if (f.use) {
         if (j.b.ntot <= 0) return launch_fwd(j, f);
-        e = cudaMemsetAsync(j.f_atm, 0, 3 * (size_t)j.b.ntot * sizeof(double), j.st);
-        if (e == cudaSuccess && f.lj) e = cudaMemsetAsync(j.f_lj, 0, 3 * (size_t)j.b.ntot * sizeof(double), j.st);
+        e = zero_forces(j, f.lj != 0);
         return e == cudaSuccess ? launch_fwd(j, f) : e;
     }
     if (const ProdLaunch l = atm_prod_plan(j); l.warps) {

@@ -67,10 +67,12 @@ __device__ __forceinline__ float round32(double t)
 // than its error; the FP64 pipe, which takes 16 cycles a warp instruction, is left to
 // the others.  256,000 molecules: 22 -> 8.3 us.
 __global__ void k_wrap_bin(Batch B, double* __restrict__ x, int* __restrict__ cell_of,
-                           int* __restrict__ rank, int* __restrict__ count, int* __restrict__ status)
+                           int* __restrict__ rank, int* __restrict__ count, int* __restrict__ maxocc,
+                           int* __restrict__ status)
 {
     const long long n = B.ntot;
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i < 1 + ATM_NUNIT) maxocc[i] = 0;  // (k_unit_max raises them)
     if (i >= n) return;
     const Rep& rp = B.rep[B.rep_of_mol[i]];
     double xv[3];
@@ -102,8 +104,8 @@ __global__ void k_wrap_bin(Batch B, double* __restrict__ x, int* __restrict__ ce
 }
 
 // K2: exclusive scan of the cell counts (one CTA of 1024 threads, each warp
-// owns a contiguous segment)
-__global__ void __launch_bounds__(1024) k_scan(long long ncell, const int* __restrict__ count,
+// owns a contiguous segment); the counts are left at zero
+__global__ void __launch_bounds__(1024) k_scan(long long ncell, int* __restrict__ count,
                                                int* __restrict__ start)
 {
     // warp w owns the contiguous segment [w seg, (w + 1) seg) of the cells and
@@ -160,7 +162,10 @@ __global__ void __launch_bounds__(1024) k_scan(long long ncell, const int* __res
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const long long c = c0 + 32 * u + lane;
-            if (c < hi) start[c] = carry + incl[u] - v[u];
+            if (c < hi) {
+                start[c] = carry + incl[u] - v[u];
+                count[c] = 0;  // for the next build
+            }
             carry += __shfl_sync(FULL, incl[u], 31);
         }
     }
@@ -890,16 +895,19 @@ cudaError_t launch_cell_counts(const Batch& b, double* x, int* cell_of, int* ran
                                int* maxocc, int* status, bool wide, cudaStream_t st)
 {
     const long long n = b.ntot;
-    cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int) * (size_t)b.ncell, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(maxocc, 0, (1 + ATM_NUNIT) * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    if (n > 0) k_wrap_bin<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(b, x, cell_of, rank, count, status);
+    if (n > 0) {
+        // (at least a thread for every maximum)
+        k_wrap_bin<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(b, x, cell_of, rank, count, maxocc, status);
+    } else {
+        const cudaError_t e = cudaMemsetAsync(maxocc, 0, (1 + ATM_NUNIT) * sizeof(int), st);
+        if (e != cudaSuccess) return e;
+    }
     k_unit_max<<<nblk(b.ncell, MD_BLOCK), MD_BLOCK, 0, st>>>(b, count, wide ? 1 : 0, maxocc);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cell_sort(const Batch& b, const double* x, const int* cell_of, const int* rank,
-                             const int* count, int* start, int* list, int* perm, double* xl, float* xl32,
+                             int* count, int* start, int* list, int* perm, double* xl, float* xl32,
                              int* cell_sorted, cudaStream_t st)
 {
     const long long n = b.ntot;

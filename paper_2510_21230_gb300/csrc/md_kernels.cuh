@@ -58,11 +58,11 @@ constexpr int MD_BLOCK = 256;
 // maxima that size the force kernels (maxocc[0] = largest cell occupancy, maxocc[1..5]
 // = largest unit of 3c01, 3c18, 3c08, 3cw, corner-anchored 3c08 (3cw's only when wide; 0
 // otherwise), maxocc[6] = of the forward lists); then the sort.  rank and list: [n] scratch,
-// rank may be perm
+// rank may be perm; count: [ncell], zero at the first build and left at zero by each
 cudaError_t launch_cell_counts(const Batch& b, double* x, int* cell_of, int* rank, int* count,
                                int* maxocc, int* status, bool wide, cudaStream_t st);
 cudaError_t launch_cell_sort(const Batch& b, const double* x, const int* cell_of, const int* rank,
-                             const int* count, int* start, int* list, int* perm, double* xl, float* xl32,
+                             int* count, int* start, int* list, int* perm, double* xl, float* xl32,
                              int* cell_sorted, cudaStream_t st);
 cudaError_t launch_lj(int prec, const LjArgs<double>& a64, const LjArgs<float>& a32,
                       cudaStream_t st);

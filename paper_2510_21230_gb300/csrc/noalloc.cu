@@ -34,7 +34,7 @@ constexpr size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct NaLayout {
     size_t rep, rep_of_cell, rep_of_mol, x, cell_of, rank, count, start, perm, cell_sorted, xl,
-        xl32, f_lj, f_atm, unit_ew, unit_cnt, unit_ew2, unit_cnt2, mol_ew, mol_cnt, ke, res, status,
+        xl32, f_lj, unit_ew, unit_cnt, unit_ew2, unit_cnt2, mol_ew, mol_cnt, ke, res, status,
         maxocc, total;
 };
 
@@ -57,8 +57,7 @@ constexpr NaLayout na_layout()
     L.cell_sorted = o; o = al256(o + NA_N * sizeof(int));
     L.xl = o;          o = al256(o + 3 * NA_N * sizeof(double));
     L.xl32 = o;        o = al256(o + 3 * NA_N * sizeof(float));
-    L.f_lj = o;        o = al256(o + 3 * NA_N * sizeof(double));
-    L.f_atm = o;       o = al256(o + 3 * NA_N * sizeof(double));
+    L.f_lj = o;        o = al256(o + 6 * NA_N * sizeof(double));  // f_atm behind it
     L.unit_ew = o;     o = al256(o + 2 * NA_C * sizeof(double));
     L.unit_cnt = o;    o = al256(o + 2 * NA_C * sizeof(unsigned long long));
     L.unit_ew2 = o;    o = al256(o + 2 * NA_C * sizeof(double));
@@ -167,7 +166,7 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     double* xl = reinterpret_cast<double*>(base + NA.xl);
     float* xl32 = reinterpret_cast<float*>(base + NA.xl32);
     double* f_lj = reinterpret_cast<double*>(base + NA.f_lj);
-    double* f_atm = reinterpret_cast<double*>(base + NA.f_atm);
+    double* f_atm = f_lj + 3 * n;  // (zeroed together)
     double* unit_ew = reinterpret_cast<double*>(base + NA.unit_ew);
     unsigned long long* unit_cnt = reinterpret_cast<unsigned long long*>(base + NA.unit_cnt);
     double* unit_ew2 = reinterpret_cast<double*>(base + NA.unit_ew2);
@@ -187,18 +186,13 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     b.ntot = n;
     b.ncell = rp.g.ncell;
 
-    // replica descriptor and positions in (the cell build wraps positions in
-    // place); replica ids, the status word and the kinetic energies start at zero
+    // replica descriptor and positions in (the cell build wraps positions in place
+    // and tests them); replica ids and kinetic energies are zero in the scratch, and
+    // nothing writes them; the status word starts at zero
     const size_t bytes3 = 3 * (size_t)n * sizeof(double);
     NA_CU(cudaMemcpyAsync(d_rep, &rp, sizeof(Rep), cudaMemcpyHostToDevice, st));
-    NA_CU(cudaMemsetAsync(rep_of_cell, 0, (size_t)b.ncell * sizeof(int), st));
-    if (n > 0) {
-        NA_CU(cudaMemsetAsync(rep_of_mol, 0, (size_t)n * sizeof(int), st));
-        NA_CU(cudaMemsetAsync(ke, 0, (size_t)n * sizeof(double), st));
-        NA_CU(cudaMemcpyAsync(x, x_dev, bytes3, cudaMemcpyDeviceToDevice, st));
-    }
+    if (n > 0) NA_CU(cudaMemcpyAsync(x, x_dev, bytes3, cudaMemcpyDeviceToDevice, st));
     NA_CU(cudaMemsetAsync(status, 0, sizeof(int), st));
-    if (n > 0) NA_CU(launch_check_finite(3 * n, x, status, st));
     NA_CU(launch_cell_counts(b, x, cell_of, perm, count, maxocc, status, false, st));
     NA_CU(launch_cell_sort(b, x, cell_of, perm, count, start, rank, perm, xl, xl32, cell_sorted, st));
     // the status word and the occupancy maxima behind it in one copy
