@@ -41,7 +41,7 @@ cudaError_t launch_atm_fwd(const FwdArgs& a, int det, int nwarps, cudaStream_t s
     if (!k) return cudaErrorInvalidValue;
     cudaError_t e = fwd_attr(a.lj, det, smem);
     if (e != cudaSuccess) return e;
-    k<<<(unsigned)((a.run > 1 ? a.nruns : a.b.ncell) * a.split), 32 * nwarps, smem, s>>>(a);
+    launch_after(k, (a.run > 1 ? a.nruns : a.b.ncell) * a.split, 32 * nwarps, smem, s, a);
     return cudaGetLastError();
 }
 

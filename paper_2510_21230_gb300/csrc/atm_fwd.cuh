@@ -592,6 +592,7 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
 template <int LJ, bool DET>
 __global__ void __launch_bounds__(32 * FWD_MAXW, 4) k_atm_fwd(const FwdArgs A)
 {
+    after_previous();
     const int b = (int)(A.split > 1 ? blockIdx.x / A.split : blockIdx.x);
     int u = b;
     if (A.run > 1) {

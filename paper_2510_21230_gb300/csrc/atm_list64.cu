@@ -111,6 +111,7 @@ __device__ __forceinline__ double sum3_64(double x, double y, double z, int lane
 // One CTA per run of base cells along x (as k_atm_fwd)
 __global__ void __launch_bounds__(32 * FWD_MAXW) k_list64(const List64Args A)
 {
+    after_previous();
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_beg[FWD_CELLS + 1];
@@ -490,8 +491,11 @@ cudaError_t launch_list64(const List64Args& a, cudaStream_t s)
     cudaError_t e = cudaFuncSetAttribute(k_list64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIST64_SMEM);
     if (e != cudaSuccess) return e;
     const long long units = a.run > 1 ? a.nruns : a.b.ncell;
-    k_list64<<<(unsigned)(units * a.split), 32 * FWD_MAXW, smem, s>>>(a);
+    launch_after(k_list64, (unsigned)(units * a.split), 32 * FWD_MAXW, smem, s, a);
     const unsigned grid = (unsigned)((a.n + 3) / 4);
+    // (not launch_after: CTAs that come while others still run pile up on the SMs that
+    // are free first, and the FP64 pipe of each SM is the bound: ten steps of the two
+    // replay systems 1,736 us so, 1,448 thus)
     k_tri64<<<grid, 128, 0, s>>>(a);
     if (a.lj == 1) k_edge64<1><<<grid, 128, 0, s>>>(a);
     else k_edge64<2><<<grid, 128, 0, s>>>(a);

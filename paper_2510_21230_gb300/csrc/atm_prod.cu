@@ -42,7 +42,7 @@ cudaError_t launch_atm_prod(int trav, const AtmArgs<R>& a, int nwarps, cudaStrea
     if (!prod_kernel<R>(trav)) return cudaErrorInvalidValue;
     cudaError_t e = prod_attr<R>(trav, (size_t)a.gcap);
     if (e != cudaSuccess) return e;
-    prod_kernel<R>(trav)<<<(unsigned)a.b.ncell, 32 * nwarps, (size_t)a.gcap, s>>>(a);
+    launch_after(prod_kernel<R>(trav), a.b.ncell, 32 * nwarps, (size_t)a.gcap, s, a);
     return cudaGetLastError();
 }
 

@@ -603,6 +603,7 @@ template <int TRAV, typename R>
 __global__ void __launch_bounds__(32 * PROD_MAXW) __maxnreg__(sizeof(R) == 8 ? 96 : 64)
     k_atm_prod(const AtmArgs<R> A)
 {
+    after_previous();
     atm_prod_unit<TRAV, R>(A, blockIdx.x);
 }
 

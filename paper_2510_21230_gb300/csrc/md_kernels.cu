@@ -70,6 +70,7 @@ __global__ void k_wrap_bin(Batch B, double* __restrict__ x, int* __restrict__ ce
                            int* __restrict__ rank, int* __restrict__ count, int* __restrict__ maxocc,
                            int* __restrict__ status)
 {
+    after_previous();
     const long long n = B.ntot;
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i < 1 + ATM_NUNIT) maxocc[i] = 0;  // (k_unit_max raises them)
@@ -108,6 +109,7 @@ __global__ void k_wrap_bin(Batch B, double* __restrict__ x, int* __restrict__ ce
 __global__ void __launch_bounds__(1024) k_scan(long long ncell, int* __restrict__ count,
                                                int* __restrict__ start)
 {
+    after_previous();
     // warp w owns the contiguous segment [w seg, (w + 1) seg) of the cells and
     // reads it 256 consecutive counts at a time (coalesced, eight loads in flight:
     // 19,683 cells 10 -> 8.4 us): its total first, then, after a scan of the 32
@@ -178,6 +180,7 @@ __global__ void __launch_bounds__(1024) k_scan(long long ncell, int* __restrict_
 // before the scan and the host can read it while the molecules are sorted.
 __global__ void k_unit_max(Batch B, const int* __restrict__ count, int wide, int* __restrict__ out)
 {
+    after_previous();
     long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     int m01 = 0, m18 = 0, m08 = 0, mw = 0, mf = 0, own = 0;
     if (c < B.ncell) {
@@ -269,6 +272,7 @@ __global__ void k_unit_classes(Batch B, const int* __restrict__ start, int trav,
 __global__ void k_scatter(long long n, const int* __restrict__ cell_of, const int* __restrict__ rank,
                           const int* __restrict__ start, int* __restrict__ list)
 {
+    after_previous();
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
     list[start[cell_of[i]] + rank[i]] = (int)i;
@@ -289,6 +293,7 @@ __global__ void __launch_bounds__(128) k_cell_order(Batch B, const double* __res
                                                     float* __restrict__ xl32,
                                                     int* __restrict__ cell_sorted)
 {
+    after_previous();
     const long long n = B.ntot;
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (e >= n) return;
@@ -357,6 +362,7 @@ constexpr int LJ_PARTS = 8, LJ_TILE = 512;
 template <typename R>
 __global__ void __launch_bounds__(LJ_BLOCK) k_lj_owner(const LjArgs<R> A)
 {
+    after_previous();
     typedef LjArith<R> Q;
     constexpr bool f64 = sizeof(R) == 8;
     constexpr unsigned FULL = 0xffffffffu;
@@ -510,6 +516,7 @@ __global__ void __launch_bounds__(256) k_kick(Batch B, const int* __restrict__ p
                                               double* __restrict__ x, double* __restrict__ v,
                                               int drift, double* __restrict__ ke)
 {
+    after_previous();
     const long long n = B.ntot;
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= n) return;
@@ -552,6 +559,7 @@ __global__ void __launch_bounds__(256) k_kick_orig(Batch B, const double* __rest
 __global__ void __launch_bounds__(256) k_kinetic(long long n, const double* __restrict__ v,
                                                  double* __restrict__ ke)
 {
+    after_previous();
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
     double k = 0.0;
@@ -581,6 +589,7 @@ __global__ void __launch_bounds__(256) k_rescale(Batch B, double* __restrict__ v
 // finiteness check of a state copied from device memory
 __global__ void k_check_finite(long long m, const double* __restrict__ a, int* __restrict__ status)
 {
+    after_previous();
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i < m && !isfinite(a[i])) atomicOr(status, ST_NONFINITE);
 }
@@ -751,6 +760,7 @@ __device__ void cell_candidates(const Grid& g, const int* st, int trav, long lon
 // replica adds the REDUCE_PARTS partial sums in a fixed tree.
 __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
 {
+    after_previous();
     __shared__ double sd[5][256];
     __shared__ unsigned long long su[4][256];
     const int tid = threadIdx.x;
@@ -825,6 +835,7 @@ __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
 // order), then a fixed shuffle tree; the order is the same for every launch
 __global__ void __launch_bounds__(128) k_final_reduce(ReduceArgs R)
 {
+    after_previous();
     static_assert(REDUCE_PARTS == 64, "two partials per lane");
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -867,6 +878,7 @@ __global__ void k_gather_forces(long long n, const int* __restrict__ perm,
                                 const double* __restrict__ f_lj, const double* __restrict__ f_atm,
                                 int which, double* __restrict__ out)
 {
+    after_previous();
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= n) return;
     int i = perm[s];
@@ -897,12 +909,12 @@ cudaError_t launch_cell_counts(const Batch& b, double* x, int* cell_of, int* ran
     const long long n = b.ntot;
     if (n > 0) {
         // (at least a thread for every maximum)
-        k_wrap_bin<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(b, x, cell_of, rank, count, maxocc, status);
+        launch_after(k_wrap_bin, nblk(n, MD_BLOCK), MD_BLOCK, 0, st, b, x, cell_of, rank, count, maxocc, status);
     } else {
         const cudaError_t e = cudaMemsetAsync(maxocc, 0, (1 + ATM_NUNIT) * sizeof(int), st);
         if (e != cudaSuccess) return e;
     }
-    k_unit_max<<<nblk(b.ncell, MD_BLOCK), MD_BLOCK, 0, st>>>(b, count, wide ? 1 : 0, maxocc);
+    launch_after(k_unit_max, nblk(b.ncell, MD_BLOCK), MD_BLOCK, 0, st, b, count, wide ? 1 : 0, maxocc);
     return cudaGetLastError();
 }
 
@@ -911,10 +923,10 @@ cudaError_t launch_cell_sort(const Batch& b, const double* x, const int* cell_of
                              int* cell_sorted, cudaStream_t st)
 {
     const long long n = b.ntot;
-    k_scan<<<1, 1024, 0, st>>>(b.ncell, count, start);
+    launch_after(k_scan, 1, 1024, 0, st, b.ncell, count, start);
     if (n > 0) {
-        k_scatter<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, cell_of, rank, start, list);
-        k_cell_order<<<nblk(n, 128), 128, 0, st>>>(b, x, cell_of, start, list, perm, xl, xl32, cell_sorted);
+        launch_after(k_scatter, nblk(n, MD_BLOCK), MD_BLOCK, 0, st, n, cell_of, rank, start, list);
+        launch_after(k_cell_order, nblk(n, 128), 128, 0, st, b, x, cell_of, start, list, perm, xl, xl32, cell_sorted);
     }
     return cudaGetLastError();
 }
@@ -935,9 +947,9 @@ cudaError_t launch_lj(int prec, const LjArgs<double>& a64, const LjArgs<float>& 
     long long n = prec == 0 ? a64.n : a32.n;
     if (n <= 0) return cudaSuccess;
     if (prec == 0)
-        k_lj_owner<double><<<(unsigned)a64.b.ncell, LJ_BLOCK, 0, st>>>(a64);
+        launch_after(k_lj_owner<double>, (unsigned)a64.b.ncell, LJ_BLOCK, 0, st, a64);
     else
-        k_lj_owner<float><<<(unsigned)a32.b.ncell, LJ_BLOCK, 0, st>>>(a32);
+        launch_after(k_lj_owner<float>, (unsigned)a32.b.ncell, LJ_BLOCK, 0, st, a32);
     return cudaGetLastError();
 }
 
@@ -945,7 +957,7 @@ cudaError_t launch_kick(const Batch& b, const int* perm, const double* f_lj, con
                         double* x, double* v, int drift, double* ke, cudaStream_t st)
 {
     if (b.ntot <= 0) return cudaSuccess;
-    k_kick<<<nblk(b.ntot, MD_BLOCK), MD_BLOCK, 0, st>>>(b, perm, f_lj, f_atm, x, v, drift, ke);
+    launch_after(k_kick, nblk(b.ntot, MD_BLOCK), MD_BLOCK, 0, st, b, perm, f_lj, f_atm, x, v, drift, ke);
     return cudaGetLastError();
 }
 
@@ -968,21 +980,21 @@ cudaError_t launch_rescale(const Batch& b, double* v, double* ke, const ResultDe
 cudaError_t launch_kinetic(long long n, const double* v, double* ke, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    k_kinetic<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, v, ke);
+    launch_after(k_kinetic, nblk(n, MD_BLOCK), MD_BLOCK, 0, st, n, v, ke);
     return cudaGetLastError();
 }
 
 cudaError_t launch_check_finite(long long m, const double* a, int* status, cudaStream_t st)
 {
     if (m <= 0) return cudaSuccess;
-    k_check_finite<<<nblk(m, MD_BLOCK), MD_BLOCK, 0, st>>>(m, a, status);
+    launch_after(k_check_finite, nblk(m, MD_BLOCK), MD_BLOCK, 0, st, m, a, status);
     return cudaGetLastError();
 }
 
 cudaError_t launch_final_reduce(const ReduceArgs& r, cudaStream_t st)
 {
-    k_partial_reduce<<<(unsigned)(r.b.R * REDUCE_PARTS), 256, 0, st>>>(r);
-    k_final_reduce<<<(unsigned)((r.b.R + 3) / 4), 128, 0, st>>>(r);
+    launch_after(k_partial_reduce, (unsigned)(r.b.R * REDUCE_PARTS), 256, 0, st, r);
+    launch_after(k_final_reduce, (unsigned)((r.b.R + 3) / 4), 128, 0, st, r);
     return cudaGetLastError();
 }
 
@@ -990,7 +1002,7 @@ cudaError_t launch_gather_forces(long long n, const int* perm, const double* f_l
                                  const double* f_atm, int which, double* out, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    k_gather_forces<<<nblk(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, perm, f_lj, f_atm, which, out);
+    launch_after(k_gather_forces, nblk(n, MD_BLOCK), MD_BLOCK, 0, st, n, perm, f_lj, f_atm, which, out);
     return cudaGetLastError();
 }
 
