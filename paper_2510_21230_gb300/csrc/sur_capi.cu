@@ -442,7 +442,8 @@ namespace {
 // (sample > 0, tensor cores: the rows are drawn in the kernel from that many)
 atm_status grad_step(atm_ctx* c, SurState* S, const float* D, const float* V, const float* T,
                      const long long* idx, long long batch, double sigma2, int update, double lr,
-                     double* loss_dev, float* grad_dev, long long sample = 0, uint64_t seed = 0)
+                     double* loss_dev, float* grad_dev, long long sample = 0, uint64_t seed = 0,
+                     bool chained = false)
 {
     const int nct = S->train_tc ? sur_grad_tc_tiles(batch) : (int)((batch + SUR_TILE - 1) / SUR_TILE);
     if (nct > S->part_cap) {
@@ -464,6 +465,7 @@ atm_status grad_step(atm_ctx* c, SurState* S, const float* D, const float* V, co
     g.S = sample;
     g.seed = seed;
     g.step = S->adam_t;
+    g.chained = chained ? 1 : 0;
     g.P = S->P;
     g.mean = S->mean;
     g.scale = S->scale;
@@ -696,7 +698,7 @@ extern "C" atm_status atm_surrogate_train(atm_ctx* c, int64_t steps, int64_t bat
             c->n_launch += 1;
         }
         atm_status s = grad_step(c, S, S->D, S->V, S->T, full ? nullptr : S->idx, B, S->sigma2, 1,
-                                 lr, S->d_loss + t, nullptr, full || !S->train_tc ? 0 : S->rows, seed);
+                                 lr, S->d_loss + t, nullptr, full || !S->train_tc ? 0 : S->rows, seed, t > 0);
         if (s != ATM_OK) return s;
     }
     if (loss) CU(cudaMemcpyAsync(loss, S->d_loss, (size_t)steps * sizeof(double), cudaMemcpyDeviceToHost, c->st));

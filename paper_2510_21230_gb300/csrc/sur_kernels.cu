@@ -895,6 +895,7 @@ __device__ __forceinline__ void pack_param(SurPacked* Pk, int k, float val)
 // gradient = sum of the CTA parts in CTA order; Adam (Kingma & Ba, Algorithm 1)
 __global__ void __launch_bounds__(64) k_sur_adam(const SurAdamArgs A)
 {
+    after_previous();
     // the parts are added in tile order, sixteen loads in flight at a time (bound
     // by their latency: 10.4 us with one, 6.8 with sixteen, 64 parts)
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1044,7 +1045,7 @@ cudaError_t launch_sur_grad(const SurGradArgs& a, int nct, cudaStream_t st)
 
 cudaError_t launch_sur_adam(const SurAdamArgs& a, cudaStream_t st)
 {
-    k_sur_adam<<<blocks_of(SUR_NP + 1, 64), 64, 0, st>>>(a);
+    launch_after(k_sur_adam, blocks_of(SUR_NP + 1, 64), 64, 0, st, a);
     return cudaGetLastError();
 }
 

@@ -106,6 +106,7 @@ struct SurGradArgs {
     // tensor-core training: S > 0 draws the rows in the kernel (sur_sample)
     unsigned long long seed;
     long long step, S;
+    int chained;              // the launch before is the Adam step (which writes no rows)
     const float* P;           // [SUR_NP] FP32 master parameters
     const float* mean;        // [32]
     const float* scale;       // [32]
