@@ -50,14 +50,39 @@ F3 = {"3c01": 109.0, "3c18": 127.0, "3c08": 127.0, "3c08a": 127.0}
 # three derivatives 26, energy 4, the two rows' sums 20 (3c01 counts a triplet
 # at each of its three owners).
 F3_FORWARD = 68.0
+# The FP64 lists: the dot product and the sides' sums 8, products, root and its
+# powers 15, the derivatives 15, three pair sums 3 (the edges' sums are per pair).
+F3_LIST64 = 41.0
+# The product rule: three squared sides 13, half sums 12, products, root and its
+# powers 14, energy 4, the derivatives 15, the forces of three molecules 24 (3c01: 9).
+F3_PRODUCT = {"3c01": 67.0, "3c18": 82.0, "3c08": 82.0, "3c08a": 82.0}
 
 
 def forward_lists(trav, trunc, prec):
     return prec == "fp32c" and trunc == "pair" and trav in ("3c01", "3c18", "3c08")
 
 
-def flops3(trav, trunc, prec):
+def lists64(trav, trunc, prec, det=False):
+    return prec == "fp64" and trunc == "pair" and trav in ("3c01", "3c18", "3c08") and not det
+
+
+def kernel_name(trav, trunc, prec, det=False):
+    """The kernel that carries an evaluation's triplets."""
+    if forward_lists(trav, trunc, prec):
+        return "k_atm_fwd"
+    if lists64(trav, trunc, prec, det):
+        return "k_tri64 (after k_list64, with k_edge64)"
+    if trunc == "product" and trav in F3_PRODUCT and not det:
+        return "k_atm_prod"
+    return "atm_owner_kernel" if trav in ("3c01", "3cw") else "atm_block_kernel"
+
+
+def flops3(trav, trunc, prec, det=False):
     """Useful flops per counted interacting triplet."""
+    if lists64(trav, trunc, prec, det):
+        return F3_LIST64 / 3.0 if trav == "3c01" else F3_LIST64
+    if trunc == "product" and trav in F3_PRODUCT and not det and prec != "surrogate":
+        return F3_PRODUCT[trav]
     if forward_lists(trav, trunc, prec):
         return F3_FORWARD / 3.0 if trav == "3c01" else F3_FORWARD
     return F3[trav]
@@ -79,7 +104,7 @@ FUSED_TRAV = ("3c08", "3c18", "3c08a")
 # capture (2197 units) scaled to 19683 units.
 KERNEL_SOURCES = ["atm3_internal.cuh", "atm_common.cuh", "atm_block.cuh", "atm_owner.cuh",
                   "atm_fp32.cu", "atm_fp64.cu", "atm_launch.cuh", "pair_masks.cu", "atm_fwd.cuh",
-                  "atm_fwd.cu"]
+                  "atm_fwd.cu", "atm_list64.cu", "atm_prod.cuh", "atm_prod.cu"]
 TRAFFIC = {("3c08", "pair", "fp32c", "liquid_n256k"): (32.43e6, "86ebe58ae46bedf4"),
            ("3c08", "pair", "fp32c", "liquid_n32k"): (3.620e6, "86ebe58ae46bedf4")}
 
@@ -370,9 +395,8 @@ def run_ours(args):
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak,
                 "traffic": traffic_for(args.trav, args.trunc, args.prec, args.workload),
-                "kernel": (("k_atm_fwd<%s,%s,%s>" if forward_lists(args.trav, args.trunc, args.prec)
-                            else "atm_owner_kernel<%s,%s,%s>" if args.trav == "3c01"
-                            else "atm_block_kernel<%s,%s,%s>") % (args.trav, args.trunc, args.prec)
+                "kernel": (kernel_name(args.trav, args.trunc, args.prec)
+                           + "<%s,%s,%s>" % (args.trav, args.trunc, args.prec)
                            + (" (LJ inside)" if fused else "")
                            + (" after k_pair_masks" if args.prec == "fp32c" and args.trunc == "pair"
                               and args.trav == "3c08a" else "")),
@@ -440,7 +464,7 @@ def run_ours(args):
             am = r["prof"]["ms_atm"] / max(1, r["prof"]["n_atm_launches"])
             # useful flops over the ATM evaluation's time, against the measured
             # FMA peak of the variant's precision
-            vflops = flops3(tv, tr, pr) * r["res"]["n_int3"]
+            vflops = flops3(tv, tr, pr, det) * r["res"]["n_int3"]
             if tv in FUSED_TRAV and tr == "pair":
                 vflops += F2_FUSED * r["res"]["n_int2"]
             if pr not in vpeak:

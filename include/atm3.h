@@ -83,19 +83,23 @@ typedef enum { ATM_TRUNC_PAIR = 0, ATM_TRUNC_PRODUCT = 1 } atm_truncation;
 
 /* Arithmetic of the force evaluation.
  *  FP64:  every decision and every force, energy and virial term in FP64.
+ *         (Pair rule of 3C01, 3C18 and 3C08, and the product rule: terms on
+ *         displacements of the wrapped positions, one rounding each.)
  *  FP32C: decisions and per-triplet arithmetic in FP32 on FP32 cell-local
  *         coordinates (every pair decision on the canonical displacement
  *         (xl_q - xl_p) + (o_q - o_p) w).  Force sums: under the pair rule 3C01,
  *         3C18 and 3C08 find the same triplets, each evaluated once at its
  *         lowest molecule i on the FP32 displacements from i; what the
  *         triplets of i put on one partner is a plain FP32 sum, and the shares
- *         of different i are added in FP64.  3C08A and the product rule of
- *         3C18 / 3C08 add each triplet's three pair scalars to per-edge FP32
- *         sums (pair rule: on the FP32-rounded unit-frame positions xl + o w),
- *         then each molecule's share of a unit is a plain FP32 sum over its
- *         edges, and the shares of different units are added in FP64; 3C01
- *         (product rule) and 3CW keep compensated (Kahan) FP32 per-lane sums
- *         of F_i, combined in FP64.  Energy and
+ *         of different i are added in FP64.  The product rule of 3C01, 3C18,
+ *         3C08 and 3C08A takes the FP32-rounded unit-frame positions xl + o w
+ *         relative to a triplet's first molecule; a unit's forces are plain
+ *         FP32 sums, those of different units are added in FP64 (3C01: per-lane
+ *         sums of F_i, combined in FP64).  The pair rule of 3C08A adds each
+ *         triplet's three pair scalars to per-edge FP32 sums on the same
+ *         positions, then each molecule's share of a unit is a plain FP32 sum
+ *         over its edges; 3CW keeps compensated (Kahan) FP32 per-lane sums of
+ *         F_i, combined in FP64.  Energy and
  *         virial: Kahan-compensated FP32 per lane, reduced in FP64.  (The
  *         deterministic mode sums the block traversals' terms in fixed
  *         point instead, see atm_set_deterministic.)
@@ -244,8 +248,10 @@ atm_status atm_get_results(atm_ctx* ctx, atm_result* out);
 /* Launch options.  persistent = 1: the ATM kernel runs as a persistent grid
  * (resident CTAs x SMs) whose CTAs take traversal units from a global counter
  * instead of one CTA per unit.  nwarps = 4 or 8 warps per 3C18/3C08 CTA (0 =
- * default); neither applies to the FP32C pair rule of 3C01, 3C18 and 3C08,
- * whose launch form follows from the system.  graph = 1: atm_step captures one step in a CUDA graph (on a
+ * default); neither applies to the pair rule of 3C01, 3C18 and 3C08 (FP64:
+ * outside the deterministic mode) and to the product rule outside the
+ * deterministic mode (3CW apart), whose launch form follows from the system.
+ * graph = 1: atm_step captures one step in a CUDA graph (on a
  * stream of its own) and replays it, with no host synchronisation between
  * steps; the graph sizes the kernels for the current largest unit plus
  * headroom (at most a quarter of it, the largest amount that keeps the
