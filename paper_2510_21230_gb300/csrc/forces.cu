@@ -79,11 +79,11 @@ cudaError_t enqueue_lj(const ForceJob& j)
     LjArgs<float> l32{};
     if (j.prec == 0) {
         l64.b = j.b; l64.n = j.b.ntot; l64.xl = j.xl; l64.xl32 = j.xl32; l64.cell_start = j.start;
-        l64.cell_sorted = j.cell_sorted; l64.fs = j.f_lj; l64.mol_ew = j.mol_ew;
+        l64.fs = j.f_lj; l64.mol_ew = j.mol_ew;
         l64.mol_cnt = j.mol_cnt;
     } else {
         l32.b = j.b; l32.n = j.b.ntot; l32.xl = j.xl32; l32.xl32 = j.xl32; l32.cell_start = j.start;
-        l32.cell_sorted = j.cell_sorted; l32.fs = j.f_lj; l32.mol_ew = j.mol_ew;
+        l32.fs = j.f_lj; l32.mol_ew = j.mol_ew;
         l32.mol_cnt = j.mol_cnt;
     }
     return launch_lj(j.prec, l64, l32, j.st);

@@ -11,7 +11,6 @@ struct LjArgs {
     const R* xl;              // sorted cell-local coordinates, SoA [3n]
     const float* xl32;        // FP32 copy (prefilter of the FP64 path)
     const int* cell_start;    // [ncell + 1]
-    const int* cell_sorted;   // [n] global cell of each sorted slot
     double* fs;               // sorted-order LJ force, SoA [3n] (fully written)
     double* mol_ew;           // [2n] per sorted molecule: half of its pair energies, virials
     unsigned* mol_cnt;        // [2n] per sorted molecule: half-shell candidates, interacting pairs
