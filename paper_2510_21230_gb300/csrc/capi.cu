@@ -205,6 +205,7 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
         }
         c->params.push_back(params[r]);
         c->reps.push_back(rp);
+        c->rc_exp = std::max(c->rc_exp, rc_exponent(rp));
         ntot += n[r];
         ncell += rp.g.ncell;
         if (ncell > (1ll << 30)) {
@@ -573,6 +574,7 @@ static bool fwd_active(const atm_ctx* c, int trav, int trunc, int prec)
     j.runs = c->d_runs;
     j.nruns = c->nruns;
     j.l64 = c->maxocc <= PM_CELL_MAX ? &c->l64 : nullptr;
+    j.rc_exp = c->rc_exp;
     j.mcap = c->unit_max[trav];
     j.x = c->x;
     return atm_uses_lists(j) || atm_prod_plan(j).warps;
@@ -641,7 +643,7 @@ static bool use_pair_masks(const atm_ctx* c, int trav, int trunc, int prec)
 void atm3::ctx_want_list64(atm_ctx* c, int trav, int trunc, int prec, int mcap)
 {
     if (prec != ATM_FP64 || trunc != ATM_TRUNC_PAIR || (trav != ATM_3C01 && trav != ATM_3C18 && trav != ATM_3C08) ||
-        c->det || !c->whole || c->n <= 0 || c->maxocc > PM_CELL_MAX)
+        c->det || !c->whole || c->n <= 0 || c->maxocc > PM_CELL_MAX || c->rc_exp > LIST64_RC_EXP)
         return;
     List64Args& l = c->l64;
     if (l.list && l.stride >= mcap) return;
@@ -742,6 +744,7 @@ atm_status atm3::ctx_enqueue_forces(atm_ctx* c, int trav, int trunc, int prec, i
     j.nruns = c->nruns;
     j.x = c->x;
     j.perm = c->perm;
+    j.rc_exp = c->rc_exp;
     if (!c->capturing) ctx_want_list64(c, trav, trunc, prec, j.mcap_fwd);
     j.l64 = c->maxocc <= PM_CELL_MAX ? &c->l64 : nullptr;
     const FwdLaunch fwd = atm_fwd_plan(j), l64 = atm_list64_plan(j);

@@ -86,6 +86,7 @@ struct atm_ctx {
     bool f_l64 = false;      // and those were the FP64 ones
     atm3::List64Args l64{};  // their buffers (first used: allocated)
     bool whole = true;       // every replica owns all its layers
+    int rc_exp = 0;          // ForceJob.rc_exp
     bool wide_cells = false;  // cell builds also size the wide traversal's 5^3 units
     // forces of the current state given by the caller (original order, total),
     // for the combination f_in_key = (traversal, truncation, precision)

@@ -3,6 +3,7 @@
 // allocation-free entry point (noalloc.cu).
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 
 #include "forces.cuh"
 
@@ -72,6 +73,8 @@ atm_status make_rep(const atm_params& p, long long n, long long mol0, long long 
     r.own_z1 = r.g.nc[2];
     return ATM_OK;
 }
+
+int rc_exponent(const Rep& r) { return std::abs(std::ilogb(r.rc)); }
 
 cudaError_t enqueue_lj(const ForceJob& j)
 {
@@ -208,12 +211,13 @@ FwdLaunch atm_fwd_plan(const ForceJob& j)
 // deterministic mode and with every cell within the bitmaps' 32 molecules:
 // forces and LJ of 32,000 molecules 0.68 ms against 1.67 ms of the block kernel
 // and 0.62 ms of the LJ kernel, of 1,000 molecules 0.06 ms against 0.87 ms of the
-// owner and LJ kernels.
+// owner and LJ kernels.  (Their first test is of FP32 squares, which hold r_c^2 to
+// full precision for r_c within 2^+-40.)
 FwdLaunch atm_list64_plan(const ForceJob& j)
 {
     FwdLaunch f;
     if (j.prec != 0 || j.trunc != 0 || (j.trav != 0 && j.trav != 1 && j.trav != 2) || !j.l64 ||
-        !j.l64->list || j.det || !j.whole || j.mcap_fwd <= 0 || j.mcap_fwd > j.l64->stride ||
+        !j.l64->list || j.det || !j.whole || j.rc_exp > LIST64_RC_EXP || j.mcap_fwd <= 0 || j.mcap_fwd > j.l64->stride ||
         j.mcap_fwd > 65535)
         return f;
     f.lj = j.lj && j.trav != 0 ? 1 : (j.lj_apart ? 2 : 0);
@@ -231,12 +235,14 @@ FwdLaunch atm_list64_plan(const ForceJob& j)
 // kernel), while a warp's tables fit beside the largest unit: faster at every size
 // measured (calls: 32,000 molecules, 3c18 FP32 3.93 -> 1.08 ms; 11,702, 3c08 FP32
 // 0.63 -> 0.50; 15,001, 3c08 FP64 3.74 -> 2.24; 20,869, 3c18 FP64 4.70 -> 2.79; 7,811,
-// 3c01 FP64 12.2 -> 3.8).
+// 3c01 FP64 12.2 -> 3.8).  FP64: for r_c within 2^+-16, where the scan's FP32
+// products of six lengths are far from the ends of their range (an r_c of 1e-9, in
+// metres, would find no triplet); the other kernels decide in FP64 what FP32 cannot.
 ProdLaunch atm_prod_plan(const ForceJob& j)
 {
     ProdLaunch l;
     if (j.trunc != 1 || j.trav < 0 || j.trav > 4 || j.trav == 3 || j.det || j.mcap < 1 || j.mcap > 65535 ||
-        (j.trav != 0 && j.mcap > ATM_MCAP_LIMIT) || (j.prec == 0 && !j.x))
+        (j.trav != 0 && j.mcap > ATM_MCAP_LIMIT) || (j.prec == 0 && (!j.x || j.rc_exp > PROD64_RC_EXP)))
         return l;
     const bool f64 = j.prec == 0;
     const long long fixed = f64 ? prod_smem<double>(j.trav, j.mcap).total : prod_smem<float>(j.trav, j.mcap).total;

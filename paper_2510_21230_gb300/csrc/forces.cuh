@@ -87,7 +87,11 @@ struct ForceJob {
     const int* perm = nullptr;
     const int* runs = nullptr;  // FwdArgs.runs and nruns of FWD_RUN cells (device)
     long long nruns = 0;
+    int rc_exp = 0;             // largest rc_exponent of the replicas
 };
+
+// distance of r_c from 1 in powers of two
+int rc_exponent(const Rep& r);
 
 // how an evaluation from forward lists is launched
 struct FwdLaunch {

@@ -44,19 +44,21 @@ __device__ __forceinline__ int bin1(double t, double w, double iw, int n, double
 }
 
 // a non-negative finite double to FP32, the mantissa cut off (integer work: a
-// conversion takes the FP64 pipe); below 2^-126 zero
+// conversion takes the FP64 pipe); below 2^-126 zero, from 2^128 infinity
 __device__ __forceinline__ float cut32(double t)
 {
     const int hi = __double2hiint(t);  // (-0: zero too)
+    if (hi >= 0x47f00000) return __int_as_float(0x7f800000);
     return hi < 0x38100000 ? 0.0f
                            : __uint_as_float(((unsigned)(hi - 0x38000000) << 3) | ((unsigned)__double2loint(t) >> 29));
 }
 
-// a double in [0, 2^127) to FP32, rounded to nearest even (integer work again)
+// a non-negative double to FP32, rounded to nearest even (integer work again,
+// where the result is a normal number below 2^127)
 __device__ __forceinline__ float round32(double t)
 {
     const unsigned long long u = (unsigned long long)__double_as_longlong(t);
-    if (u < 0x3810000000000000ull) return (float)t;
+    if (u - 0x3810000000000000ull >= 0x0fd0000000000000ull) return (float)t;
     return __uint_as_float((unsigned)((u + 0x0fffffffull + ((u >> 29) & 1ull)) >> 29) - (896u << 23));
 }
 
@@ -414,7 +416,9 @@ __global__ void __launch_bounds__(LJ_BLOCK) k_lj_owner(const LjArgs<R> A)
     const R eps24 = f64 ? (R)rp.eps24 : (R)rp.eps24f;
     const R eps48 = f64 ? (R)rp.eps48 : (R)rp.eps48f;
     const R ushift = f64 ? (R)rp.ushift : (R)rp.ushiftf;
-    const float c_hi = rp.rc2f * (1.0f + 0x1p-16f);
+    // (FP64: the band of its prefilter; a comparison that zeros, infinities and NaN of
+    // FP32 pass, so that units far from 1 are decided in FP64)
+    const float c_hi = f64 ? rp.p_hi : rp.rc2f * (1.0f + 0x1p-16f);
     const int part = tid % LJ_PARTS;
     auto stage = [&](int base) {
         for (int k = tid; k < LJ_TILE && base + k < M; k += LJ_BLOCK) {
@@ -458,7 +462,8 @@ __global__ void __launch_bounds__(LJ_BLOCK) k_lj_owner(const LjArgs<R> A)
                 for (int b = 0; b < m; b++) {
                     const float4 p = S4[c0 + part + b * LJ_PARTS];
                     const float dx = p.x - fx0, dy = p.y - fy0, dz = p.z - fz0;
-                    if (dx * dx + dy * dy + dz * dz < c_hi) hit |= 1u << b;
+                    const float c = dx * dx + dy * dy + dz * dz;
+                    if (f64 ? !(c > c_hi) : c < c_hi) hit |= 1u << b;
                 }
                 while (hit) {
                     const int q = c0 + part + (__ffs(hit) - 1) * LJ_PARTS, t = base + q;
@@ -664,8 +669,9 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(Batch B, const double* _
         int cx, cy, cz;
         cell_coords(rp.g, cg - rp.cell0, cx, cy, cz);
         const float wx = rp.wf[0], wy = rp.wf[1], wz = rp.wf[2];
-        // squares up to 12 w^2 from rounded coordinates: within 2^-18 of that
-        const float c_hi = (float)rmax2 * (1.0f + 0x1p-20f) + 0x1p-14f * (wx * wx + wy * wy + wz * wz);
+        // squares up to 12 w^2 from rounded coordinates: within 2^-18 of that (or of the
+        // least FP32 numbers; zeros, infinities and NaN pass the test below)
+        const float c_hi = (float)rmax2 * (1.0f + 0x1p-20f) + 0x1p-14f * (wx * wx + wy * wy + wz * wz) + 0x1p-144f;
         const float xs = xl32[s], ys = xl32[n + s], zs = xl32[2 * n + s];
         int dx = 0, dy = 0, dz = 0, q0 = 0, q1 = 0;
         if (lane < 14) {
@@ -684,7 +690,7 @@ __global__ void __launch_bounds__(32 * RDF_WARPS) k_rdf(Batch B, const double* _
                 bool keep = false;
                 if (q < e) {
                     const float ex = (xl32[q] - xs) + ox, ey = (xl32[n + q] - ys) + oy, ez = (xl32[2 * n + q] - zs) + oz;
-                    keep = ex * ex + ey * ey + ez * ez < c_hi;
+                    keep = !(ex * ex + ey * ey + ez * ez > c_hi);
                 }
                 const unsigned m = __ballot_sync(FULL, keep);
                 if (m == 0) continue;

@@ -236,6 +236,7 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     j.perm = perm;
     j.lj_apart = true;
     j.nruns = fwd_runs_of(rp.g);
+    j.rc_exp = rc_exponent(rp);
     const FwdLaunch fwd = atm_fwd_plan(j);
     if (fwd.lj != 2) NA_CU(enqueue_lj(j));
     bool capacity = false;
