@@ -25,53 +25,11 @@
 #include "atm3_internal.cuh"
 #include "forces.cuh"
 #include "md_kernels.cuh"
+#include "noalloc_layout.cuh"
 
 using namespace atm3;
 
 namespace {
-
-constexpr size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
-
-struct NaLayout {
-    size_t rep, rep_of_cell, rep_of_mol, x, cell_of, rank, count, start, perm, cell_sorted, xl,
-        xl32, f_lj, unit_ew, unit_cnt, unit_ew2, unit_cnt2, mol_ew, mol_cnt, ke, res, status,
-        maxocc, total;
-};
-
-constexpr long long NA_N = ATM_NOALLOC_MAX_N;
-constexpr long long NA_C = ATM_NOALLOC_MAX_CELLS;
-
-constexpr NaLayout na_layout()
-{
-    NaLayout L{};
-    size_t o = 0;
-    L.rep = o;         o = al256(o + sizeof(Rep));
-    L.rep_of_cell = o; o = al256(o + NA_C * sizeof(int));
-    L.rep_of_mol = o;  o = al256(o + NA_N * sizeof(int));
-    L.x = o;           o = al256(o + 3 * NA_N * sizeof(double));
-    L.cell_of = o;     o = al256(o + NA_N * sizeof(int));
-    L.rank = o;        o = al256(o + NA_N * sizeof(int));
-    L.count = o;       o = al256(o + NA_C * sizeof(int));
-    L.start = o;       o = al256(o + (NA_C + 1) * sizeof(int));
-    L.perm = o;        o = al256(o + NA_N * sizeof(int));
-    L.cell_sorted = o; o = al256(o + NA_N * sizeof(int));
-    L.xl = o;          o = al256(o + 3 * NA_N * sizeof(double));
-    L.xl32 = o;        o = al256(o + 3 * NA_N * sizeof(float));
-    L.f_lj = o;        o = al256(o + 6 * NA_N * sizeof(double));  // f_atm behind it
-    L.unit_ew = o;     o = al256(o + 2 * NA_C * sizeof(double));
-    L.unit_cnt = o;    o = al256(o + 2 * NA_C * sizeof(unsigned long long));
-    L.unit_ew2 = o;    o = al256(o + 2 * NA_C * sizeof(double));
-    L.unit_cnt2 = o;   o = al256(o + 2 * NA_C * sizeof(unsigned long long));
-    L.mol_ew = o;      o = al256(o + 2 * NA_N * sizeof(double));
-    L.mol_cnt = o;     o = al256(o + 2 * NA_N * sizeof(unsigned));
-    L.ke = o;          o = al256(o + NA_N * sizeof(double));
-    L.res = o;         o = al256(o + (1 + REDUCE_PARTS) * sizeof(ResultDev));
-    L.status = o;      o = al256(o + sizeof(int));
-    L.maxocc = o;      o = al256(o + (1 + ATM_NUNIT) * sizeof(int));
-    L.total = o;
-    return L;
-}
-constexpr NaLayout NA = na_layout();
 
 // the scratch array (about 7.8 MB at the limits above)
 __device__ __align__(256) unsigned char g_na_scratch[NA.total];
@@ -154,12 +112,13 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     NA_CU(na_scratch(p->device, &base));
     cudaStream_t st = (cudaStream_t)p->cuda_stream;
     Rep* d_rep = reinterpret_cast<Rep*>(base + NA.rep);
-    int* rep_of_cell = reinterpret_cast<int*>(base + NA.rep_of_cell);
-    int* rep_of_mol = reinterpret_cast<int*>(base + NA.rep_of_mol);
+    const NaZero Z = na_zero(n, rp.g.ncell);
+    int* rep_of_cell = reinterpret_cast<int*>(base + Z.rep_of_cell);
+    int* rep_of_mol = reinterpret_cast<int*>(base + Z.rep_of_mol);
     double* x = reinterpret_cast<double*>(base + NA.x);
     int* cell_of = reinterpret_cast<int*>(base + NA.cell_of);
     int* rank = reinterpret_cast<int*>(base + NA.rank);
-    int* count = reinterpret_cast<int*>(base + NA.count);
+    int* count = reinterpret_cast<int*>(base + Z.count);
     int* start = reinterpret_cast<int*>(base + NA.start);
     int* perm = reinterpret_cast<int*>(base + NA.perm);
     int* cell_sorted = reinterpret_cast<int*>(base + NA.cell_sorted);
@@ -173,10 +132,10 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     unsigned long long* unit_cnt2 = reinterpret_cast<unsigned long long*>(base + NA.unit_cnt2);
     double* mol_ew = reinterpret_cast<double*>(base + NA.mol_ew);
     unsigned* mol_cnt = reinterpret_cast<unsigned*>(base + NA.mol_cnt);
-    double* ke = reinterpret_cast<double*>(base + NA.ke);
+    double* ke = reinterpret_cast<double*>(base + Z.ke);
     ResultDev* res = reinterpret_cast<ResultDev*>(base + NA.res);
-    int* status = reinterpret_cast<int*>(base + NA.status);
-    int* maxocc = reinterpret_cast<int*>(base + NA.maxocc);
+    int* status = reinterpret_cast<int*>(base + Z.status);
+    int* maxocc = reinterpret_cast<int*>(base + Z.maxocc);
 
     Batch b;
     b.rep = d_rep;
@@ -187,16 +146,15 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     b.ncell = rp.g.ncell;
 
     // replica descriptor and positions in (the cell build wraps positions in place
-    // and tests them); replica ids and kinetic energies are zero in the scratch, and
-    // nothing writes them; the status word starts at zero
+    // and tests them); what must start at zero
     const size_t bytes3 = 3 * (size_t)n * sizeof(double);
     NA_CU(cudaMemcpyAsync(d_rep, &rp, sizeof(Rep), cudaMemcpyHostToDevice, st));
     if (n > 0) NA_CU(cudaMemcpyAsync(x, x_dev, bytes3, cudaMemcpyDeviceToDevice, st));
-    NA_CU(cudaMemsetAsync(status, 0, sizeof(int), st));
+    NA_CU(cudaMemsetAsync(base + NA.zero, 0, Z.end - NA.zero, st));
     NA_CU(launch_cell_counts(b, x, cell_of, perm, count, maxocc, status, false, st));
     NA_CU(launch_cell_sort(b, x, cell_of, perm, count, start, rank, perm, xl, xl32, cell_sorted, st));
     // the status word and the occupancy maxima behind it in one copy
-    constexpr size_t OCC = (NA.maxocc - NA.status) / sizeof(int);
+    constexpr size_t OCC = NA_ALIGN / sizeof(int);
     int hbuf[OCC + 1 + ATM_NUNIT] = {};
     NA_CU(cudaMemcpyAsync(hbuf, status, sizeof(hbuf), cudaMemcpyDeviceToHost, st));
     const int* hocc = hbuf + OCC;
@@ -264,13 +222,13 @@ static atm_status noalloc_run(const atm_params* p, int64_t n, const double* x_de
     NA_CU(launch_final_reduce(r, st));
     if (n > 0) NA_CU(launch_gather_forces(n, perm, f_lj, f_atm, 0, f_dev, st));
     // the result and the status word behind the partial sums in one copy
-    alignas(ResultDev) unsigned char hout[NA.status - NA.res + sizeof(int)];
+    alignas(ResultDev) unsigned char hout[NA.zero - NA.res + sizeof(int)];
     NA_CU(cudaMemcpyAsync(hout, res, sizeof(hout), cudaMemcpyDeviceToHost, st));
     NA_CU(cudaStreamSynchronize(st));
     ResultDev hres;
     int hstat;
     memcpy(&hres, hout, sizeof(hres));
-    memcpy(&hstat, hout + (NA.status - NA.res), sizeof(hstat));
+    memcpy(&hstat, hout + (NA.zero - NA.res), sizeof(hstat));
     if (hstat & ST_NONFINITE) return ATM_E_NONFINITE;
     if (hstat & ST_CAPACITY) return ATM_E_CAPACITY;
     if (out) {
