@@ -526,7 +526,12 @@ extern "C" atm_status atm_build_cells(atm_ctx* c)
     if (!c) return ATM_E_INVALID;
     if (!c->have_x) return ctx_fail(c, ATM_E_STATE, "no state set");
     CU(cudaSetDevice(c->device));
-    return enqueue_cells(c);
+    const atm_status s = enqueue_cells(c);
+    if (s != ATM_OK) return s;
+    // (a step goes on while the molecules are sorted; this call returns with the
+    // stream idle)
+    CU(cudaStreamSynchronize(c->st));
+    return ATM_OK;
 }
 
 extern "C" atm_status atm_get_cells(atm_ctx* c, int32_t* cell_of, int32_t* cell_start,
