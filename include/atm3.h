@@ -136,7 +136,15 @@ typedef struct {
 
 typedef struct atm_ctx atm_ctx;
 
-/* Create a context for n molecules (n >= 0).  Allocates every device buffer.
+/* Create a context for n molecules (n >= 0).  Allocates every device buffer but
+ * those that only some contexts use, which the first call that uses them
+ * allocates and the context keeps: the surrogate's, and the lists of the FP64 pair
+ * rule of 3C01, 3C18 and 3C08 (whole systems, cells of at most 32 molecules,
+ * outside the deterministic mode): 16 bytes for every molecule of the fullest 18
+ * cells and an eighth more, and 160 bytes, a molecule (5 KB in a liquid at density
+ * 0.8), allocated anew when units outgrow that.  Where they would take more than
+ * 16 GiB, or the device has no room for them, the same evaluations run without
+ * them, slower.
  * Errors: INVALID, BOX_TOO_SMALL, CUDA.  *out is NULL on failure. */
 atm_status atm_create(const atm_params* params, int64_t n, atm_ctx** out);
 

@@ -651,17 +651,17 @@ void atm3::ctx_want_list64(atm_ctx* c, int trav, int trunc, int prec, int mcap)
         c->det || !c->whole || c->n <= 0 || c->maxocc > PM_CELL_MAX || c->rc_exp > LIST64_RC_EXP)
         return;
     List64Args& l = c->l64;
-    if (l.list && l.stride >= mcap) return;
-    // a row for any list of an 18-cell unit, with room for units to grow
-    const long long stride = ((mcap + mcap / 8 + 15) / 8) * 8;
+    const long long stride = list64_rows_wanted(c->n, l.list ? l.stride : 0, c->l64_refused, mcap);
+    if (stride == 0) return;  // (there, or not to be had: the plan looks at the stride)
     const size_t rows = (size_t)c->n * (size_t)stride;
-    cudaStreamSynchronize(c->st);
-    drop_graph(c);
-    void* old[] = {l.list, l.G, l.place, l.count, l.mol_w3, l.mol_n3};
-    for (void* p : old)
-        if (p) cudaFree(p);
-    l = List64Args{};
-    if (rows * 16 > ((size_t)16 << 30)) return;  // (the block kernel then)
+    if (l.list) {
+        cudaStreamSynchronize(c->st);
+        drop_graph(c);  // (its launches hold the old buffers)
+        void* old[] = {l.list, l.G, l.place, l.count, l.mol_w3, l.mol_n3};
+        for (void* p : old)
+            if (p) cudaFree(p);
+        l = List64Args{};
+    }
     bool ok = cudaMalloc((void**)&l.list, rows * sizeof(uint2)) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&l.G, (rows + PM_CELL_MAX) * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&l.place, 18 * (size_t)c->n * sizeof(uint2)) == cudaSuccess;
@@ -674,6 +674,7 @@ void atm3::ctx_want_list64(atm_ctx* c, int trav, int trunc, int prec, int mcap)
         for (void* p : got)
             if (p) cudaFree(p);
         l = List64Args{};
+        c->l64_refused = stride;
         return;
     }
     l.stride = stride;

@@ -84,7 +84,8 @@ struct atm_ctx {
     int f_split = 1;         // partial sums per cell in the unit arrays
     bool f_fwd = false;      // the current forces came from forward lists
     bool f_l64 = false;      // and those were the FP64 ones
-    atm3::List64Args l64{};  // their buffers (first used: allocated)
+    atm3::List64Args l64{};  // their buffers (allocated by the first evaluation that takes them)
+    long long l64_refused = 0;  // entries a row that could not be allocated (0: none so far)
     bool whole = true;       // every replica owns all its layers
     int rc_exp = 0;          // ForceJob.rc_exp
     bool wide_cells = false;  // cell builds also size the wide traversal's 5^3 units

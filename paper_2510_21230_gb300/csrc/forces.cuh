@@ -102,6 +102,22 @@ struct FwdLaunch {
 FwdLaunch atm_fwd_plan(const ForceJob& j);
 // the same for the FP64 lists (lj 1 or 2)
 FwdLaunch atm_list64_plan(const ForceJob& j);
+// The FP64 lists' buffers: a row of list64_stride(mcap) entries of 16 bytes for each
+// of n molecules, any list of an 18-cell unit of mcap molecules with an eighth for
+// units to grow (a liquid at density 0.8: 310 entries, 5 KB a molecule), up to 16 GiB.
+constexpr unsigned long long LIST64_MAX_BYTES = 16ull << 30;
+inline long long list64_stride(int mcap) { return ((long long)mcap + mcap / 8 + 15) / 8 * 8; }
+// the entries a row to allocate now for units of mcap molecules; 0: rows of `have`
+// hold them, or they are beyond the limit, or rows of `refused` or fewer entries
+// could not be had before (neither is tried again at every evaluation, and rows
+// that are there stay)
+inline long long list64_rows_wanted(long long n, long long have, long long refused, int mcap)
+{
+    if (have >= mcap) return 0;
+    const long long s = list64_stride(mcap);
+    if ((unsigned long long)n * (unsigned long long)s * 16 > LIST64_MAX_BYTES) return 0;
+    return refused > 0 && s >= refused ? 0 : s;
+}
 // the product-rule kernel's warps per CTA (0: the job does not take it) and bytes
 // of shared memory
 struct ProdLaunch {
