@@ -89,7 +89,26 @@ struct Frame64 {
         dy = (x[n + o] - yi) + sy;
         dz = (x[2 * n + o] - zi) + sz;
     }
+    // d(g -> h) of two partners in 18-cell slots s and t: exact for a close pair
+    __device__ __forceinline__ void between(int g, int s, int h, int t, double& dx, double& dy, double& dz) const
+    {
+        int ox, oy, oz, px, py, pz;
+        slot18(s, ox, oy, oz);
+        slot18(t, px, py, pz);
+        const long long o = perm[g], p = perm[h];
+        auto image = [](int c, int m) { return c < 0 ? -1 : (c >= m ? 1 : 0); };
+        dx = (x[p] - x[o]) + (double)(image(cx + px, nx) - image(cx + ox, nx)) * L0;
+        dy = (x[n + p] - x[n + o]) + (double)(image(cy + py, ny) - image(cy + oy, ny)) * L1;
+        dz = (x[2 * n + p] - x[2 * n + o]) + (double)(image(cz + pz, nz) - image(cz + oz, nz)) * L2;
+    }
 };
+
+// c is below an eighth of the larger of a and b (by the bits of their high words: no
+// FP64 instruction; a negative c is)
+__device__ __forceinline__ bool small_side(double a, double b, double c)
+{
+    return __double2hiint(c) + (3 << 20) < max(__double2hiint(a), __double2hiint(b));
+}
 
 // v (one per lane and component) summed over the warp: lane 8 d holds component d
 __device__ __forceinline__ double sum3_64(double x, double y, double z, int lane)
@@ -335,8 +354,22 @@ __global__ void __launch_bounds__(128) k_tri64(const List64Args A)
         double xj, yj, zj, a, xk, yk, zk, b;
         row64(j, xj, yj, zj, a);
         row64(k, xk, yk, zk, b);
-        const double m = xj * xk + yj * yk + zj * zk;
-        const double x = a - m, y = b - m, c = x + y;
+        double m = xj * xk + yj * yk + zj * zk;
+        double x = a - m, y = b - m, c = x + y;
+        // c by cancellation keeps fewer digits than the rows have where it is below
+        // a + b by more than 16 (measured against extended precision on triangles of a
+        // liquid's sides: rms force error 4.1e-15 above that line, where displacements
+        // of three roundings each and their differences give 4.8e-15; 1.4e-13 at 1/256);
+        // there it comes from the two positions (1.6e-15).  A liquid has next to none.
+        if (small_side(a, b, c)) {
+            const uint2 ej = meta(j), ek = meta(k);
+            double ex, ey, ez;
+            F.between((int)ej.x, (int)(ej.y & 0xffu), (int)ek.x, (int)(ek.y & 0xffu), ex, ey, ez);
+            c = ex * ex + ey * ey + ez * ez;
+            x = -(xj * ex + yj * ey + zj * ez);
+            y = c - x;
+            m = a - x;
+        }
         const double bc = b * c, ac = a * c, ab = a * b;
         const double q = rsqrt(a * bc);
         const double q2 = q * q;

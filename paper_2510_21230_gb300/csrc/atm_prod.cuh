@@ -37,8 +37,8 @@
 //
 // 32,000 molecules at density 0.8, 3c18, FP32: 0.86 ms (the block kernel: 3.69), issue
 // 55 % and the shared-memory reductions 50 % busy; with rows in staging order and hits
-// queued it took 2.1.  15,001 at 0.7, 3c08, FP64: 1.80 ms (3.36), FP64 pipe 83 % busy,
-// 64 instructions a triplet of which 38 are its arithmetic.  7,811, 3c01, FP64: 3.8 ms
+// queued it took 2.1.  15,001 at 0.7, 3c08, FP64: 1.90 ms (3.36), bound by
+// the FP64 pipe, 69 instructions a triplet of which 43 are its arithmetic.  7,811, 3c01, FP64: 3.8 ms
 // a call (12.2).
 //
 // Decisions.  Squares from unit-frame positions are within 2.4e-4 (relative) of
@@ -291,8 +291,10 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
             const double2 Q0 = rows64[2 * j], Q1 = rows64[2 * j + 1], V0 = rows64[2 * k], V1 = rows64[2 * k + 1];
             const double qx = Q0.x, qy = Q0.y, qz = Q1.x, a = Q1.y;
             const double rx = V0.x, ry = V0.y, rz = V1.x, b = V1.y;
-            const double m = qx * rx + qy * ry + qz * rz;
-            const double x = a - m, y = b - m, c = x + y;
+            // (the third side from the difference of the rows: a + b - 2 q.r would lose the
+            // digits of a side short against the others, of which this rule has many)
+            const double ex = rx - qx, ey = ry - qy, ez = rz - qz, c = ex * ex + ey * ey + ez * ez;
+            const double x = -(qx * ex + qy * ey + qz * ez), y = c - x, m = a - x;
             const double abc = a * (b * c);
             if (abc > rp.rc6 * (1.0 - 0x1p-30)) {
                 if (abc > rp.rc6 * (1.0 + 0x1p-30)) return;
@@ -311,13 +313,13 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
                 fpy = fma(ga, qy, fma(gb, ry, fpy));
                 fpz = fma(ga, qz, fma(gb, rz, fpz));
                 if constexpr (!OWNER) {
-                    const double ex = gc * (rx - qx), ey = gc * (ry - qy), ez = gc * (rz - qz);
-                    atomicAdd(F + 3 * q, fma(-ga, qx, ex));
-                    atomicAdd(F + 3 * q + 1, fma(-ga, qy, ey));
-                    atomicAdd(F + 3 * q + 2, fma(-ga, qz, ez));
-                    atomicAdd(F + 3 * r, -fma(gb, rx, ex));
-                    atomicAdd(F + 3 * r + 1, -fma(gb, ry, ey));
-                    atomicAdd(F + 3 * r + 2, -fma(gb, rz, ez));
+                    const double gx = gc * ex, gy = gc * ey, gz = gc * ez;
+                    atomicAdd(F + 3 * q, fma(-ga, qx, gx));
+                    atomicAdd(F + 3 * q + 1, fma(-ga, qy, gy));
+                    atomicAdd(F + 3 * q + 2, fma(-ga, qz, gz));
+                    atomicAdd(F + 3 * r, -fma(gb, rx, gx));
+                    atomicAdd(F + 3 * r + 1, -fma(gb, ry, gy));
+                    atomicAdd(F + 3 * r + 2, -fma(gb, rz, gz));
                 }
             }
         }
