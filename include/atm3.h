@@ -92,10 +92,10 @@ typedef enum { ATM_TRUNC_PAIR = 0, ATM_TRUNC_PRODUCT = 1 } atm_truncation;
  *         lowest molecule i on the FP32 displacements from i; what the
  *         triplets of i put on one partner is a plain FP32 sum, and the shares
  *         of different i are added in FP64.  The product rule of 3C01, 3C18,
- *         3C08 and 3C08A takes the FP32-rounded unit-frame positions xl + o w
- *         relative to a triplet's first molecule; a unit's forces are plain
- *         FP32 sums, those of different units are added in FP64 (3C01: per-lane
- *         sums of F_i, combined in FP64).  The pair rule of 3C08A adds each
+ *         3C08 and 3C08A takes the canonical displacements from a triplet's
+ *         first molecule; a unit's forces are plain FP32 sums, those of
+ *         different units are added in FP64 (3C01: compensated (Kahan) FP32
+ *         per-lane sums of F_i, combined in FP64).  The pair rule of 3C08A adds each
  *         triplet's three pair scalars to per-edge FP32 sums on the same
  *         positions, then each molecule's share of a unit is a plain FP32 sum
  *         over its edges; 3CW keeps compensated (Kahan) FP32 per-lane sums of

@@ -19,12 +19,14 @@
 // that hold the farther row have hits alike: the longest list of 32 lanes is 1.5
 // to 1.8 of their mean; with rows in staging order, or lanes that hold the
 // nearer row, it is 3 to 5.)  In a liquid 3c18 tests 24 % of its candidates.
-//   FP32  a lane evaluates its own hits, one a turn; nothing is queued, r's force
+//   FP32  what is evaluated are the canonical displacements of the rows, as in the owner
+//         kernel (unit-frame positions are rounded at 2 w: rms force error up to a
+//         sixth more).  A lane evaluates its own hits, one a turn; nothing is queued, r's force
 //         stays in registers and p's too, q's goes to shared memory by three
 //         reductions.  A lane begins at its own bit of a word, and eight copies of
 //         the forces take the lanes in turn, for the far rows of a p share their
 //         few near ones (32,000 molecules, 3c18: 1.72 ms with one, 0.88 with four,
-//         0.86 with eight).
+//         0.86 with eight).  3c01 adds p's force compensated.
 //   FP64  an instruction takes the FP64 pipe as long for one lane as for 32, so
 //         hits are queued, one a lane and turn, and evaluated 32 at a time; lanes
 //         hold the nearer row there (hits of one batch meet fewer equal rows).
@@ -282,6 +284,7 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
     Sum<R> esum;
     unsigned nint = 0;
     R fpx, fpy, fpz;  // force on p: the lane's share
+    Sum<float> fox, foy, foz;  // the same of 3c01 in FP32, compensated
     int qn = 0;
     R* Fl = F + (lane & (NF - 1));  // the lane's copy of the forces
     // FP64: one queued hit, two rows of p, per lane
@@ -340,6 +343,15 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
             py = X[M + p];
             pz = X[2 * M + p];
         }
+        // FP32: the rows that are evaluated are the canonical displacements
+        float lx = 0.0f, ly = 0.0f, lz = 0.0f;
+        const int sp = __float_as_int(P.w);
+        if constexpr (!F64) {
+            const long long g = sidx[p];
+            lx = A.xl[g];
+            ly = A.xl[n + g];
+            lz = A.xl[2 * n + g];
+        }
         const int first = OWNER ? 0 : p + 1;
         bins[lane] = 0;
         __syncwarp();
@@ -369,8 +381,17 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
                 to[2] = V.y;
                 to[4] = V.z;
                 to[6] = b;
-                if constexpr (!F64) rows4[k] = make_float4(V.x, V.y, V.z, __int_as_float(t));
-                else rid[k] = (unsigned short)t;
+                if constexpr (!F64) {
+                    const long long g = sidx[t];
+                    const int s = __float_as_int(S4[t].w);
+                    float dx, dy, dz;
+                    canon_disp<float>(lx, ly, lz, A.xl[g], A.xl[n + g], A.xl[2 * n + g], s_off[s][0] - s_off[sp][0],
+                                      s_off[s][1] - s_off[sp][1], s_off[s][2] - s_off[sp][2], rp.wf[0], rp.wf[1],
+                                      rp.wf[2], dx, dy, dz);
+                    rows4[k] = make_float4(dx, dy, dz, __int_as_float(t));
+                } else {
+                    rid[k] = (unsigned short)t;
+                }
                 if constexpr (F64) {
                     const double dx = X[t] - px, dy = X[M + t] - py, dz = X[2 * M + t] - pz;
                     rows64[2 * k] = make_double2(dx, dy);
@@ -401,6 +422,7 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
         }
         __syncwarp();
         fpx = fpy = fpz = R(0);
+        fox = foy = foz = Sum<float>();
         // ---- 32 rows, a row per lane: FP32 with the rows before, FP64 with those after
         for (int r0 = 0; r0 < np; r0 += 32) {
             const int r = r0 + lane;
@@ -408,11 +430,19 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
             float Vx = 0.0f, Vy = 0.0f, Vz = 0.0f, b = 0.0f;
             int ri = p, v = 0;
             if (own) {
-                const float* vr = rows + 8 * (r >> 1) + (r & 1);
-                Vx = vr[0];
-                Vy = vr[2];
-                Vz = vr[4];
-                b = vr[6];
+                if constexpr (F64) {
+                    const float* vr = rows + 8 * (r >> 1) + (r & 1);
+                    Vx = vr[0];
+                    Vy = vr[2];
+                    Vz = vr[4];
+                    b = vr[6];
+                } else {
+                    const float4 V = rows4[r];
+                    Vx = V.x;
+                    Vy = V.y;
+                    Vz = V.z;
+                    b = Vx * Vx + Vy * Vy + Vz * Vz;
+                }
                 ri = staged(r);
             }
             if constexpr (TRAV == 2) v = __float_as_int(P.w) & __float_as_int(S4[ri].w);
@@ -506,11 +536,15 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
                             prod_terms<float>(a, b, c, fmaf(0.5f, c, -w), fmaf(0.5f, c, w), fmaf(-0.5f, c, t), uu, ga,
                                               gb, gc);
                             esum.add(uu);
-                            gr += gb;
-                            fpx = fmaf(ga, Q.x, fpx);
-                            fpy = fmaf(ga, Q.y, fpy);
-                            fpz = fmaf(ga, Q.z, fpz);
-                            if constexpr (!OWNER) {
+                            if constexpr (OWNER) {
+                                fox.add(fmaf(ga, Q.x, gb * Vx));
+                                foy.add(fmaf(ga, Q.y, gb * Vy));
+                                foz.add(fmaf(ga, Q.z, gb * Vz));
+                            } else {
+                                gr += gb;
+                                fpx = fmaf(ga, Q.x, fpx);
+                                fpy = fmaf(ga, Q.y, fpy);
+                                fpz = fmaf(ga, Q.z, fpz);
                                 const float gx = gc * ex, gy = gc * ey, gz = gc * ez;
                                 frx += gx;
                                 fry += gy;
@@ -523,15 +557,13 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
                         __syncwarp();
                     }
                 }
-                if (own) {
+                if (own && !OWNER) {
                     fpx = fmaf(gr, Vx, fpx);
                     fpy = fmaf(gr, Vy, fpy);
                     fpz = fmaf(gr, Vz, fpz);
-                    if constexpr (!OWNER) {
-                        atomicAdd(Fl + 3 * NF * ri, -fmaf(gr, Vx, frx));
-                        atomicAdd(Fl + 3 * NF * ri + NF, -fmaf(gr, Vy, fry));
-                        atomicAdd(Fl + 3 * NF * ri + 2 * NF, -fmaf(gr, Vz, frz));
-                    }
+                    atomicAdd(Fl + 3 * NF * ri, -fmaf(gr, Vx, frx));
+                    atomicAdd(Fl + 3 * NF * ri + NF, -fmaf(gr, Vy, fry));
+                    atomicAdd(Fl + 3 * NF * ri + 2 * NF, -fmaf(gr, Vz, frz));
                 }
             }
         }
@@ -542,6 +574,11 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
         if constexpr (!TABLE) {
             using W = std::conditional_t<OWNER, double, R>;
             W f0 = fpx, f1 = fpy, f2 = fpz;
+            if constexpr (OWNER && !F64) {
+                f0 = fox.get();
+                f1 = foy.get();
+                f2 = foz.get();
+            }
             for (int o = 16; o > 0; o >>= 1) {
                 f0 += __shfl_down_sync(FULL, f0, o);
                 f1 += __shfl_down_sync(FULL, f1, o);
