@@ -90,8 +90,8 @@ typedef enum { ATM_TRUNC_PAIR = 0, ATM_TRUNC_PRODUCT = 1 } atm_truncation;
  *         (xl_q - xl_p) + (o_q - o_p) w).  Force sums: under the pair rule 3C01,
  *         3C18 and 3C08 find the same triplets, each evaluated once at its
  *         lowest molecule i on the FP32 displacements from i; what the
- *         triplets of i put on one partner is a plain FP32 sum, and the shares
- *         of different i are added in FP64.  The product rule of 3C01, 3C18,
+ *         triplets of i put on one partner is a plain FP32 sum (3C01:
+ *         compensated), and the shares of different i are added in FP64.  The product rule of 3C01, 3C18,
  *         3C08 and 3C08A takes the canonical displacements from a triplet's
  *         first molecule; a unit's forces are plain FP32 sums, those of
  *         different units are added in FP64 (3C01: compensated (Kahan) FP32

@@ -27,9 +27,12 @@
 //     kernel spends 37 % of its time on expanding edges into triangles and
 //     4 % on its atomics).  Row k's share of a pair goes to lane k by two shuffles:
 //     with g_e = 2 du/d(r_e^2) the force on j is
-//         sum_k g_jk (d_k - d_j) - G_ij d_j = V_j - (H_j + G_ij) d_j,
-//     V_j = sum_k g_jk d_k and H_j = sum_k g_jk, and that on i is
-//     sum_j G_ij d_j; all of it stays in registers.
+//         V_j - G_ij d_j,   V_j = sum_k g_jk (d_k - d_j),
+//     and that on i is sum_j G_ij d_j; all of it stays in registers.  (V_j as
+//     sum_k g_jk d_k - d_j sum_k g_jk is an operation less a pair, but cancels
+//     where j and k are close: rms force error of the arithmetic 2.9e-7 against 2.7e-7.)
+//     3c01 compensates these sums, as the owner kernel does (2.6e-7): 32,000
+//     molecules 111 -> 126 us, 438 in the owner kernel.
 //     The third side comes from the rows, |d_k - d_j|^2: within 2.2e-6
 //     (relative to r_c^2) of the canonical square (five FP32 roundings of
 //     values up to 4/3 r_c per component, in both), so outside a band of
@@ -92,22 +95,55 @@ __device__ __forceinline__ void fwd_add_pair(float& s, float& r, float s2, float
     s = t;
 }
 
-// v summed over the warp, for x, y and z at once: lane 8 d of the result holds
-// component d (d < 3)
-__device__ __forceinline__ float fwd_sum3(float x, float y, float z, int lane)
+// x, y, z and w summed over the warp: lane 8 d of the result holds component d
+__device__ __forceinline__ float fwd_sum4(float x, float y, float z, float w, int lane)
 {
     const unsigned FULL = 0xffffffffu;
     const bool b4 = lane & 16, b3 = lane & 8;
-    float k0 = b4 ? z : x, k1 = b4 ? 0.0f : y;
+    float k0 = b4 ? z : x, k1 = b4 ? w : y;
     k0 += __shfl_xor_sync(FULL, b4 ? x : z, 16);
-    k1 += __shfl_xor_sync(FULL, b4 ? y : 0.0f, 16);
+    k1 += __shfl_xor_sync(FULL, b4 ? y : w, 16);
     float k = b3 ? k1 : k0;
     k += __shfl_xor_sync(FULL, b3 ? k0 : k1, 8);
     for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(FULL, k, o);
     return k;
 }
 
-template <int LJ, bool DET>
+// the same in float pairs
+__device__ __forceinline__ float fwd_sum4_pair(float x, float y, float z, float w, int lane)
+{
+    const unsigned FULL = 0xffffffffu;
+    const bool b4 = lane & 16, b3 = lane & 8;
+    float k0 = b4 ? z : x, k1 = b4 ? w : y, r0 = 0.0f, r1 = 0.0f;
+    fwd_add_pair(k0, r0, __shfl_xor_sync(FULL, b4 ? x : z, 16), 0.0f);
+    fwd_add_pair(k1, r1, __shfl_xor_sync(FULL, b4 ? y : w, 16), 0.0f);
+    float k = b3 ? k1 : k0, r = b3 ? r1 : r0;
+    const float s2 = __shfl_xor_sync(FULL, b3 ? k0 : k1, 8), t2 = __shfl_xor_sync(FULL, b3 ? r0 : r1, 8);
+    fwd_add_pair(k, r, s2, t2);
+    for (int o = 4; o > 0; o >>= 1) {
+        const float s = __shfl_xor_sync(FULL, k, o), t = __shfl_xor_sync(FULL, r, o);
+        fwd_add_pair(k, r, s, t);
+    }
+    return k + r;
+}
+
+// sums of a list row: plain FP32, or (COMP) compensated
+template <bool COMP>
+struct FwdSum {
+    float s = 0.f;
+    __device__ __forceinline__ void fma(float a, float b) { s = fmaf(a, b, s); }
+    __device__ __forceinline__ void add(float v) { s += v; }
+    __device__ __forceinline__ float get() const { return s; }
+};
+template <>
+struct FwdSum<true> {
+    Sum<float> k;
+    __device__ __forceinline__ void fma(float a, float b) { k.add(__fmul_rn(a, b)); }
+    __device__ __forceinline__ void add(float v) { k.add(v); }
+    __device__ __forceinline__ float get() const { return __fsub_rn(k.s, k.c); }
+};
+
+template <int LJ, bool DET, bool COMP>
 __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, const int part)
 {
     constexpr unsigned FULL = 0xffffffffu;
@@ -235,6 +271,10 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
         return d;
     };
 
+    // (the owner kernel that 3c01 had combined its lanes' shares in FP64)
+    auto sum4 = [&](float x, float y, float z, float w) -> float {
+        return COMP ? fwd_sum4_pair(x, y, z, w, lane) : fwd_sum4(x, y, z, w, lane);
+    };
     Sum<float> esum, e2sum, w2sum;
     unsigned nint = 0, n2 = 0;
     const int M0 = s_base[len];
@@ -298,17 +338,15 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
 
         float fix = 0.f, fiy = 0.f, fiz = 0.f;  // force on i, this lane's share
         float fjx = 0.f, fjy = 0.f, fjz = 0.f;  // (LJ apart) its LJ part
-        // sums of the lane's row j: V = sum g_jk d_k, H = sum g_jk, G = g_ij,
-        // all over 3 nu
+        // sums of the lane's row j: V = sum g_jk (d_k - d_j), G = g_ij, over 3 nu
         struct RowSum {
-            float Vx = 0.f, Vy = 0.f, Vz = 0.f, H = 0.f, G = 0.f;
-            __device__ __forceinline__ void add(float gi, float gjk, const float4& d)
+            FwdSum<COMP> Vx, Vy, Vz, G;
+            __device__ __forceinline__ void add(float gi, float gjk, float ex, float ey, float ez)
             {
-                G += gi;
-                H += gjk;
-                Vx = fmaf(gjk, d.x, Vx);
-                Vy = fmaf(gjk, d.y, Vy);
-                Vz = fmaf(gjk, d.z, Vz);
+                G.add(gi);
+                Vx.fma(gjk, ex);
+                Vy.fma(gjk, ey);
+                Vz.fma(gjk, ez);
             }
         };
         float es = 0.f;
@@ -316,11 +354,11 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
         // and x = (a + c - b) / 2, y = (b + c - a) / 2, m = (a + b - c) / 2,
         //     2 du/da = 3 nu q^5 (a y - x m - b c (1 + 5 x y m q^2)), cyclic,
         //     u = nu q^3 (1 + 3 x y m q^2), q = (a b c)^(-1/2).
-        // decide(c): the third side's decision
+        // decide(c): the third side's decision; e = d_k - d_j
         auto triangle = [&](const float4& Dj, const float4& Dk, auto decide, float& ga, float& gb,
-                            float& gc) {
+                            float& gc, float& ex, float& ey, float& ez) {
             const float a = Dj.w, b = Dk.w;
-            const float ex = Dk.x - Dj.x, ey = Dk.y - Dj.y, ez = Dk.z - Dj.z;
+            ex = Dk.x - Dj.x, ey = Dk.y - Dj.y, ez = Dk.z - Dj.z;
             const float c = ex * ex + ey * ey + ez * ez;
             const bool keep = decide(c);
             nint += keep ? 1u : 0u;
@@ -342,8 +380,7 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
         const float nu3 = 3.0f * rp.nuf;
         auto finish = [&](const float4& D, int t, const RowSum& R, bool first) {
             const int g = __float_as_int(S4[t].w);
-            float G = nu3 * R.G;
-            const float H = nu3 * R.H;
+            float G = nu3 * R.G.get();
             if (LJ && first) {
                 // LJ pair scalar of (i, j): F_i = g d(i -> j); the LJ kernel's
                 // expressions on the same displacement
@@ -369,10 +406,9 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
                     G -= fw;
                 }
             }
-            const float f = H + G;
-            add(0, g, fmaf(-f, D.x, nu3 * R.Vx));
-            add(1, g, fmaf(-f, D.y, nu3 * R.Vy));
-            add(2, g, fmaf(-f, D.z, nu3 * R.Vz));
+            add(0, g, fmaf(-G, D.x, nu3 * R.Vx.get()));
+            add(1, g, fmaf(-G, D.y, nu3 * R.Vy.get()));
+            add(2, g, fmaf(-G, D.z, nu3 * R.Vz.get()));
             fix = fmaf(G, D.x, fix);
             fiy = fmaf(G, D.y, fiy);
             fiz = fmaf(G, D.z, fiz);
@@ -410,14 +446,14 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
             };
             auto shift = [&](int s, bool ok) {
                 const float4 Dk = up[s], Ds = down[-s];
-                float ga, gb, gc;
-                triangle(Dj, Dk, [&](float c) { return near(c, ok); }, ga, gb, gc);
-                R.add(ga, gc, Dk);
+                float ga, gb, gc, ex, ey, ez;
+                triangle(Dj, Dk, [&](float c) { return near(c, ok); }, ga, gb, gc, ex, ey, ez);
+                R.add(ga, gc, ex, ey, ez);
                 // (unsigned: a negative lane - s is the larger)
                 const unsigned src = min((unsigned)(lane - s), (unsigned)(lane - s + h));
                 gb = __shfl_sync(FULL, gb, (int)src);
                 gc = __shfl_sync(FULL, gc, (int)src);
-                R.add(gb, gc, Ds);
+                R.add(gb, gc, Ds.x - Dj.x, Ds.y - Dj.y, Ds.z - Dj.z);
             };
             const int odd = (h - 1) >> 1;
 #pragma unroll 2
@@ -428,32 +464,30 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
 #pragma unroll 1
                 for (int e = 0; e < nextra; e++) {
                     // row 32 + e with the 32 rows, then with the extra ones before it
-                    float sx = 0.f, sy = 0.f, sz = 0.f, sg = 0.f, sh = 0.f;
+                    FwdSum<COMP> sx, sy, sz, sg;
                     const float4 Dk = list[64 + e];
 #pragma unroll 1
                     for (int pass = 0; pass < 2; pass++) {
                         const float4 D = pass ? De : Dj;
-                        float ga, gb, gc;
-                        triangle(D, Dk, [&](float c) { return near(c, pass ? lane < e : true); }, ga, gb, gc);
-                        if (pass) RE.add(ga, gc, Dk);
-                        else R.add(ga, gc, Dk);
-                        sg += gb;
-                        sh += gc;
-                        sx = fmaf(gc, D.x, sx);
-                        sy = fmaf(gc, D.y, sy);
-                        sz = fmaf(gc, D.z, sz);
+                        float ga, gb, gc, ex, ey, ez;
+                        triangle(D, Dk, [&](float c) { return near(c, pass ? lane < e : true); }, ga, gb, gc, ex, ey,
+                                 ez);
+                        if (pass) RE.add(ga, gc, ex, ey, ez);
+                        else R.add(ga, gc, ex, ey, ez);
+                        sg.add(gb);
+                        sx.fma(gc, ex);
+                        sy.fma(gc, ey);
+                        sz.fma(gc, ez);
                         if (e == 0) break;
                     }
-                    const float v = fwd_sum3(sx, sy, sz, lane), w = fwd_sum3(sg, sh, 0.f, lane);
+                    const float v = sum4(sx.get(), sy.get(), sz.get(), sg.get());
                     const float vx = __shfl_sync(FULL, v, 0), vy = __shfl_sync(FULL, v, 8),
-                                vz = __shfl_sync(FULL, v, 16);
-                    const float wg = __shfl_sync(FULL, w, 0), wh = __shfl_sync(FULL, w, 8);
+                                vz = __shfl_sync(FULL, v, 16), vg = __shfl_sync(FULL, v, 24);
                     if (lane == e) {
-                        RE.Vx += vx;
-                        RE.Vy += vy;
-                        RE.Vz += vz;
-                        RE.G += wg;
-                        RE.H += wh;
+                        RE.Vx.add(-vx);
+                        RE.Vy.add(-vy);
+                        RE.Vz.add(-vz);
+                        RE.G.add(vg);
                     }
                 }
             }
@@ -495,26 +529,27 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
 #pragma unroll 1
                 for (int K = J; K < np; K += h) {
                     RowSum RK;
+                    const float4 Dl = row(K + l0);
                     int k = l0, src = l0;
 #pragma unroll 1
                     for (int s = 0; s < (K == J ? (h >> 1) + 1 : h); s++) {
                         if (K > J || s > 0) {
                             const float4 Dk = row(K + k), Ds = row(J + src);
                             const bool ok = own && K + k < np && !(K == J && 2 * s == h && lane >= s);
-                            float ga, gb, gc;
+                            float ga, gb, gc, ex, ey, ez;
                             triangle(Dj, Dk, [&](float c) {
                                 if (!ok || c >= c_hi) return false;
                                 return c < c_lo || canon(P4[tj], P4[lidx[K + k]]).w < rc2;
-                            }, ga, gb, gc);
-                            R.add(ga, gc, Dk);
+                            }, ga, gb, gc, ex, ey, ez);
+                            R.add(ga, gc, ex, ey, ez);
                             gb = __shfl_sync(FULL, gb, src);
                             gc = __shfl_sync(FULL, gc, src);
-                            RK.add(gb, gc, Ds);
+                            RK.add(gb, gc, Ds.x - Dl.x, Ds.y - Dl.y, Ds.z - Dl.z);
                         }
                         k = k + 1 == h ? 0 : k + 1;
                         src = src == 0 ? h - 1 : src - 1;
                     }
-                    if (lane < h && K + lane < np) finish(row(K + lane), lidx[K + lane], RK, false);
+                    if (lane < h && K + lane < np) finish(Dl, lidx[K + lane], RK, false);
                 }
                 if (own) {
                     finish(Dj, tj, R, true);
@@ -525,10 +560,10 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
         }
         const int d = lane >> 3;
         const bool mine = lane < 24 && (lane & 7) == 0;
-        const float fi = fwd_sum3(fix, fiy, fiz, lane);
+        const float fi = sum4(fix, fiy, fiz, 0.0f);
         if (mine) add(d, __float_as_int(si.w), fi);
         if (LJ == 2) {
-            const float fj = fwd_sum3(fjx, fjy, fjz, lane);
+            const float fj = fwd_sum4(fjx, fjy, fjz, 0.0f, lane);
             if (mine) atomicAdd(A.fs_lj + d * n + __float_as_int(si.w), fwd_widen(fj));
         }
         __syncwarp();  // the list is read to the end before the next one is written
@@ -588,9 +623,10 @@ __device__ __forceinline__ void atm_fwd_unit(const FwdArgs& A, const int u, cons
 
 // One CTA per run of base cells along x (one cell per run, and split > 1 CTAs
 // dealt its molecules, for systems of too few cells to fill the GPU).
-// LJ: 0 none, 1 into fs, 2 apart
-template <int LJ, bool DET>
-__global__ void __launch_bounds__(32 * FWD_MAXW, 4) k_atm_fwd(const FwdArgs A)
+// LJ: 0 none, 1 into fs, 2 apart.  COMP (3c01): compensated sums, at three CTAs
+// to an SM for their registers
+template <int LJ, bool DET, bool COMP>
+__global__ void __launch_bounds__(32 * FWD_MAXW, COMP ? 3 : 4) k_atm_fwd(const FwdArgs A)
 {
     after_previous();
     const int b = (int)(A.split > 1 ? blockIdx.x / A.split : blockIdx.x);
@@ -603,7 +639,7 @@ __global__ void __launch_bounds__(32 * FWD_MAXW, 4) k_atm_fwd(const FwdArgs A)
             u = b / nseg * nx + b % nseg * A.run;
         }
     }
-    atm_fwd_unit<LJ, DET>(A, u, A.split > 1 ? (int)(blockIdx.x % A.split) : 0);
+    atm_fwd_unit<LJ, DET, COMP>(A, u, A.split > 1 ? (int)(blockIdx.x % A.split) : 0);
 }
 
 }  // namespace atm3

@@ -182,6 +182,7 @@ FwdLaunch atm_fwd_plan(const ForceJob& j)
     // LJ apart only for whole systems (in a domain the LJ kernel gives owned
     // molecules their complete force) and in floating point
     f.lj = j.lj && j.trav != 0 ? 1 : (j.lj_apart && j.whole && !j.det ? 2 : 0);
+    if (j.trav == 0 && f.lj != 2) return f;  // (no kernel of this form)
     // eight warps and a run of four cells per CTA; one cell, and several CTAs per
     // cell, while the grid would leave SMs without enough warps
     const long long sms = j.sms > 0 ? j.sms : 148, occ = (j.b.ntot + j.b.ncell - 1) / j.b.ncell;
