@@ -87,21 +87,23 @@ typedef enum { ATM_TRUNC_PAIR = 0, ATM_TRUNC_PRODUCT = 1 } atm_truncation;
  *         displacements of the wrapped positions, one rounding each.)
  *  FP32C: decisions and per-triplet arithmetic in FP32 on FP32 cell-local
  *         coordinates (every pair decision on the canonical displacement
- *         (xl_q - xl_p) + (o_q - o_p) w).  Force sums: under the pair rule 3C01,
- *         3C18 and 3C08 find the same triplets, each evaluated once at its
- *         lowest molecule i on the FP32 displacements from i; what the
- *         triplets of i put on one partner is a plain FP32 sum (3C01:
- *         compensated), and the shares of different i are added in FP64.  The product rule of 3C01, 3C18,
- *         3C08 and 3C08A takes the canonical displacements from a triplet's
- *         first molecule; a unit's forces are plain FP32 sums, those of
- *         different units are added in FP64 (3C01: compensated (Kahan) FP32
- *         per-lane sums of F_i, combined in FP64).  The pair rule of 3C08A adds each
- *         triplet's three pair scalars to per-edge FP32 sums on the same
- *         positions, then each molecule's share of a unit is a plain FP32 sum
- *         over its edges; 3CW keeps compensated (Kahan) FP32 per-lane sums of
- *         F_i, combined in FP64.  Energy and
- *         virial: Kahan-compensated FP32 per lane, reduced in FP64.  (The
- *         deterministic mode sums the block traversals' terms in fixed
+ *         (xl_q - xl_p) + (o_q - o_p) w).
+ *         Force sums: under the pair rule 3C01, 3C18 and 3C08 find the same
+ *         triplets, each evaluated once at its lowest molecule i on the canonical
+ *         displacements from i; what the triplets of i put on one partner is a
+ *         plain FP32 sum (3C01: compensated), and the shares of different i are
+ *         added in FP64.  The product rule of 3C01, 3C18, 3C08 and 3C08A takes the
+ *         canonical displacements from a triplet's first molecule; a unit's forces
+ *         are plain FP32 sums, those of different units are added in FP64 (3C01:
+ *         compensated (Kahan) FP32 per-lane sums of F_i, combined in FP64).  The
+ *         pair rule of 3C08A takes the FP32-rounded unit-frame positions xl + o w and
+ *         adds each triplet's three pair scalars to per-edge FP32 sums, then each
+ *         molecule's share of a unit is a plain FP32 sum over its edges; 3CW keeps
+ *         compensated FP32 per-lane sums of F_i, combined in FP64.
+ *         Energy: compensated FP32 per lane, reduced in FP64.  Virial: likewise, or
+ *         9 times the energy (u is homogeneous of degree -9 in the distances: 3C01,
+ *         3C18 and 3C08 under the pair rule, and the product rule).
+ *         (The deterministic mode sums the block traversals' terms in fixed
  *         point instead, see atm_set_deterministic.)
  *  SURROGATE: the ATM force comes from the learned per-molecule model below
  *         (atm_surrogate_*), not from triplets; LJ runs in FP32.  The model
