@@ -1012,7 +1012,8 @@ static atm_status run_graph_steps(atm_ctx* c, int nsteps, int trav, int trunc, i
     if (fwd) cls[0] = 1;
     const int mcap = graph_mcap(c, trav, trunc, prec, nwarps);
     const int key[10] = {trav, trunc, prec, mcap, fwd ? graph_mcap_fwd(c) : 0,
-                        persistent + 2 * nwarps + 64 * (use_pair_masks(c, trav, trunc, prec) ? 1 : 0),
+                        persistent + 2 * nwarps + 64 * (use_pair_masks(c, trav, trunc, prec) ? 1 : 0) +
+                            128 * (prec == ATM_SURROGATE && c->maxocc > 32 ? 1 : 0),
                         cls[0], cls[1], cls[2], edge_capacity(c, trav, trunc)};
     if (!c->graph || memcmp(key, c->graph_key, sizeof(key)) != 0) {
         drop_graph(c);

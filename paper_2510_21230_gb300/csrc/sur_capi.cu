@@ -201,6 +201,7 @@ atm_status sur_args(atm_ctx* c, SurState* S, SurForceArgs& a)
     a.vb = S->vb;
     a.status = c->d_status;
     a.sms = c->sms;
+    a.maxocc = c->maxocc;
     return ATM_OK;
 }
 

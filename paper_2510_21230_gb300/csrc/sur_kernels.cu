@@ -181,21 +181,25 @@ __global__ void __launch_bounds__(256) k_sur_xyz4(long long n, const float* __re
 // recorded as one bit of its cell's word (cheap, so lanes in different cells
 // diverge little; the lanes of one cell read the same rows); (B) the thread
 // walks its set bits and accumulates the descriptor terms, so the expensive
-// part keeps every lane busy.  A cell of more than 32 molecules: one direct
-// pass.  With LJ the same neighbours give the FP32 LJ pair force, energy,
-// virial and counts of the molecule (the decisions and arithmetic of the FP32
-// LJ kernel, so no separate LJ pass is needed).  Mode 0 writes the normalised
+// part keeps every lane busy.  BIG (the last cell build met cells of more than 32
+// molecules: up to 4/3 r_c wide, three to a box, a liquid has them): another
+// 16 bits a cell (40 replicas of 700 at density 0.85: 177 us an evaluation, 308
+// with direct passes).  A cell of more than those 48: one direct pass.  With LJ
+// the same neighbours give the FP32 LJ pair force, energy, virial and counts of
+// the molecule (the decisions and arithmetic of the FP32 LJ kernel, so no separate
+// LJ pass is needed).  Mode 0 writes the normalised
 // bfloat16 input row and the vectors for the MLP kernel; mode 1 appends the raw
 // descriptors, vectors and the current ATM force to the data set.  The words
 // are cell-major (cell t of thread i at t * SUR_BLOCK + i), free of bank
 // conflicts.  Bound by instruction issue; a word per cell instead of one bit
 // string over the 27 cells takes the tables of cell ends and offsets and their
 // search per neighbour away: 256,000 molecules 317 -> 265 us.
-template <bool LJ>
+template <bool LJ, bool BIG>
 __global__ void __launch_bounds__(SUR_BLOCK, 5) k_sur_desc(const SurForceArgs A)
 {
     __shared__ unsigned mask[27 * SUR_BLOCK];
     __shared__ int s_q0[27 * SUR_BLOCK];  // first molecule of the cell
+    __shared__ unsigned short mask2[BIG ? 27 * SUR_BLOCK : 1];
     __shared__ float4 s_off[27];          // cell offset
     if (threadIdx.x < 27) {
         int dx, dy, dz;
@@ -255,29 +259,55 @@ __global__ void __launch_bounds__(SUR_BLOCK, 5) k_sur_desc(const SurForceArgs A)
             if (t > 13) lj_cand += (unsigned)cnt;
             if (t == 13) lj_cand += (unsigned)(q0 + cnt - 1 - (int)s);
         }
-        crowded = crowded || cnt > 32;
+        crowded = crowded || cnt > (BIG ? 48 : 32);
         const float sx = (float)dx * rp.wf[0], sy = (float)dy * rp.wf[1], sz = (float)dz * rp.wf[2];
         unsigned word = 0u;
         const float4* row = x4 + q0;
+        const int first = BIG ? min(cnt, 32) : cnt;
 #pragma unroll 4
-        for (int j = 0; j < cnt; j++) {
+        for (int j = 0; j < first; j++) {
             float ex, ey, ez;
             const float r2 = dist2(row[j], sx, sy, sz, ex, ey, ez);
             word |= (r2 < kc.rc2 ? 1u : 0u) << (j & 31);
         }
-        if (t == 13) word &= ~(1u << (((int)s - q0) & 31));  // (the molecule itself)
+        const int self = t == 13 ? (int)s - q0 : -1;  // (the molecule itself)
+        if (self >= 0 && (!BIG || self < 32)) word &= ~(1u << (self & 31));
         mask[t * SUR_BLOCK + tid] = word;
+        if constexpr (BIG) {
+            word = 0u;
+#pragma unroll 4
+            for (int j = 32; j < min(cnt, 48); j++) {
+                float ex, ey, ez;
+                const float r2 = dist2(row[j], sx, sy, sz, ex, ey, ez);
+                word |= (r2 < kc.rc2 ? 1u : 0u) << (j - 32);
+            }
+            if (self >= 32) word &= ~(1u << (self & 31));
+            mask2[t * SUR_BLOCK + tid] = (unsigned short)word;
+        }
         s_q0[t * SUR_BLOCK + tid] = q0;
     }
     if (!crowded) {
         // (B) one iteration per set bit (not per word), so every lane runs as many
         // iterations as it has neighbours
         int t = -1, q0 = 0;
-        unsigned bits = 0u;
+        unsigned bits = 0u, second = 0u;
         for (;;) {
-            while (bits == 0u && ++t < 27) bits = mask[t * SUR_BLOCK + tid];
+            while (bits == 0u) {
+                if (BIG && second != 0u) {
+                    bits = second;
+                    second = 0u;
+                    q0 += 32;
+                    break;
+                }
+                if (++t >= 27) break;
+                bits = mask[t * SUR_BLOCK + tid];
+                if constexpr (BIG) {
+                    second = mask2[t * SUR_BLOCK + tid];
+                    q0 = s_q0[t * SUR_BLOCK + tid];
+                }
+            }
             if (bits == 0u) break;
-            q0 = s_q0[t * SUR_BLOCK + tid];
+            if constexpr (!BIG) q0 = s_q0[t * SUR_BLOCK + tid];
             const int q = q0 + __ffs(bits) - 1;
             bits &= bits - 1u;
             const float4 o = s_off[t];
@@ -1016,10 +1046,9 @@ cudaError_t launch_sur_forces(const SurForceArgs& a, cudaStream_t st)
                                  a.sms, st);
     }
     k_sur_xyz4<<<blocks_of(a.n, 256), 256, 0, st>>>(a.n, a.xl32, a.xl4);
-    if (a.f_lj)
-        k_sur_desc<true><<<blocks_of(a.n, SUR_BLOCK), SUR_BLOCK, 0, st>>>(a);
-    else
-        k_sur_desc<false><<<blocks_of(a.n, SUR_BLOCK), SUR_BLOCK, 0, st>>>(a);
+    void (*const desc)(const SurForceArgs) = a.maxocc > 32 ? (a.f_lj ? k_sur_desc<true, true> : k_sur_desc<false, true>)
+                                                            : (a.f_lj ? k_sur_desc<true, false> : k_sur_desc<false, false>);
+    desc<<<blocks_of(a.n, SUR_BLOCK), SUR_BLOCK, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || a.mode != 0) return e;
     return launch_sur_mlp_tc(a.n, nullptr, a.xb, a.vb, a.model, nullptr, nullptr, a.f_atm, a.status,

@@ -85,6 +85,7 @@ struct SurForceArgs {
     unsigned* mol_cnt;        // [2n] half-shell candidates, visits
     int* status;              // device status word (ST_TIMEOUT)
     int sms;                  // SMs of the device (persistent MLP grid)
+    int maxocc;               // largest cell of the last build (chooses the kernel only)
     // mode 1 (collect): raw descriptors, vectors and the current f_atm as the
     // training target, rows [row0, row0 + n) of the data set (sorted order)
     float* d_out;             // [.][32]
