@@ -763,8 +763,12 @@ __device__ void cell_candidates(const Grid& g, const int* st, int trav, long lon
 // Two-level reduction in a fixed order (the same sums for the same partials).  Level 1: CTA
 // (r, k) sums the k-th of REDUCE_PARTS equal slices of replica r's units and
 // molecules (thread-strided, then a fixed tree).  Level 2: one warp per
-// replica adds the REDUCE_PARTS partial sums in a fixed tree.
-__global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
+// replica adds the REDUCE_PARTS partial sums in a fixed tree.  CAND: with the
+// candidates of the cells (apart, for their registers).  With many replicas the FP64 pipe
+// bounds it, 16 cycles a warp instruction: 240 replicas of 480 molecules 53 us (249 with
+// a division in every thread and whole trees for slices of a few), 90 to 100 with CAND.
+template <bool CAND>
+__global__ void __launch_bounds__(256, CAND ? 4 : 5) k_partial_reduce(ReduceArgs R)
 {
     after_previous();
     __shared__ double sd[5][256];
@@ -791,7 +795,7 @@ __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
             v2 += R.unit_cnt2[2 * q + 1];
         }
     }
-    if (R.cand_trav >= 0) {
+    if constexpr (CAND) {
         const long long cc = (rp.g.ncell + REDUCE_PARTS - 1) / REDUCE_PARTS;
         const long long l1 = min(rp.g.ncell, (k + 1) * cc);
         for (long long q = k * cc + tid; q < l1; q += 256)
@@ -812,30 +816,31 @@ __global__ void __launch_bounds__(256) k_partial_reduce(ReduceArgs R)
         }
         ke += R.ke[q];
     }
-    if (R.mol_w3) e3 = w3 / 9.0;  // u is homogeneous of degree -9 in the distances
     sd[0][tid] = e2; sd[1][tid] = e3; sd[2][tid] = w2; sd[3][tid] = w3; sd[4][tid] = ke;
     su[0][tid] = c3; su[1][tid] = i3; su[2][tid] = c2; su[3][tid] = v2;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (tid < o) {
-            for (int k = 0; k < 5; k++) sd[k][tid] += sd[k][tid + o];
-            for (int k = 0; k < 4; k++) su[k][tid] += su[k][tid + o];
+    // a warp to a quantity: the tree over halves, quarters, .. of the 256 (in that
+    // order; of slices of up to 32 the other threads have zeros)
+    const bool few = max(cu, cm) <= 32;  // (and the cells: no more than units)
+    const int lane = tid & 31;
+    double* out = reinterpret_cast<double*>(R.part + blockIdx.x);  // e2, e3, w2, w3, ekin; the counts
+    auto tree = [&](auto* v) {
+        auto half = [&](int t) { return v[t] + v[t + 128]; };
+        auto x = few ? v[lane] : (half(lane) + half(lane + 64)) + (half(lane + 32) + half(lane + 96));
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        return x;
+    };
+    for (int q = tid >> 5; q < 9; q += 8) {
+        if (q < 5) {
+            const double x = tree(sd[q]);
+            if (lane == 0) out[q] = x;
+        } else {
+            const unsigned long long x = tree(su[q - 5]);
+            if (lane == 0) reinterpret_cast<unsigned long long*>(out)[q] = x;
         }
-        __syncthreads();
-    }
-    if (tid == 0) {
-        ResultDev* p = R.part + blockIdx.x;
-        p->e2 = sd[0][0];
-        p->e3 = sd[1][0];
-        p->w2 = sd[2][0];
-        p->w3 = sd[3][0];
-        p->ekin = sd[4][0];
-        p->n_cand3 = su[0][0];
-        p->n_int3 = su[1][0];
-        p->n_cand2 = su[2][0];
-        p->n_int2 = su[3][0];
     }
 }
+static_assert(sizeof(ResultDev) == 72, "nine quantities in their order");
 
 // one warp per replica: lane k holds partials k and k + 32 (added in that
 // order), then a fixed shuffle tree; the order is the same for every launch
@@ -867,7 +872,9 @@ __global__ void __launch_bounds__(128) k_final_reduce(ReduceArgs R)
     if (lane == 0) {
         ResultDev t;
         t.e2 = e2;
-        t.e3 = e3;
+        // u is homogeneous of degree -9 in the distances (divided here, once a replica:
+        // beside the partial sums it took 1 us of an SM's FP64 pipe a CTA)
+        t.e3 = R.mol_w3 ? w3 / 9.0 : e3;
         t.w2 = w2;
         t.w3 = w3;
         t.ekin = ek;
@@ -999,7 +1006,8 @@ cudaError_t launch_check_finite(long long m, const double* a, int* status, cudaS
 
 cudaError_t launch_final_reduce(const ReduceArgs& r, cudaStream_t st)
 {
-    launch_after(k_partial_reduce, (unsigned)(r.b.R * REDUCE_PARTS), 256, 0, st, r);
+    launch_after(r.cand_trav >= 0 ? k_partial_reduce<true> : k_partial_reduce<false>, (unsigned)(r.b.R * REDUCE_PARTS),
+                 256, 0, st, r);
     launch_after(k_final_reduce, (unsigned)((r.b.R + 3) / 4), 128, 0, st, r);
     return cudaGetLastError();
 }
