@@ -245,6 +245,9 @@ struct AtmArgs {
 // FP64 evaluations that test in FP32 first: largest rc_exponent
 constexpr int LIST64_RC_EXP = 40, PROD64_RC_EXP = 16;
 
+// 3c01 in FP64: smallest largest unit of the product-rule kernel
+constexpr int PROD64_OWNER_MIN = 48;
+
 constexpr int PROD_MAXW = 16;  // most warps of a product-rule CTA
 
 constexpr int PROD_COPIES = 8;  // of the FP32 forces

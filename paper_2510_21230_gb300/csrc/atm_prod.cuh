@@ -156,6 +156,15 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
         store_zero();
         return;
     }
+    if (Mp == 0 || M < 3) {  // no triplet, and no candidate but of other corners' anchored sets
+        if (warp == 0) {
+            const unsigned long long cand =
+                OWNER ? (lane == 0 ? unit_candidates<TRAV, S>(s_beg) : 0ull) : unit_candidates_warp<TRAV, S>(s_beg);
+            store_zero();
+            if (tid == 0) A.unit_cnt[2 * u] = cand;
+        }
+        return;
+    }
     const ProdSmem plan = prod_smem<R>(TRAV, M);
     float4* S4 = reinterpret_cast<float4*>(smem + plan.off_frame);  // unit-frame position, slot
     double* X = reinterpret_cast<double*>(smem + plan.off_x);       // FP64: unit-frame positions, SoA

@@ -233,17 +233,21 @@ FwdLaunch atm_list64_plan(const ForceJob& j)
 
 // The product rule of 3c01, 3c18, 3c08 and 3c08a outside the deterministic mode (its
 // sums are fixed-point, in the block kernel, or in a fixed order, in the owner
-// kernel), while a warp's tables fit beside the largest unit: faster at every size
-// measured (calls: 32,000 molecules, 3c18 FP32 3.93 -> 1.08 ms; 11,702, 3c08 FP32
-// 0.63 -> 0.50; 15,001, 3c08 FP64 3.74 -> 2.24; 20,869, 3c18 FP64 4.70 -> 2.79; 7,811,
-// 3c01 FP64 12.2 -> 3.8).  FP64: for r_c within 2^+-16, where the scan's FP32
-// products of six lengths are far from the ends of their range (an r_c of 1e-9, in
-// metres, would find no triplet); the other kernels decide in FP64 what FP32 cannot.
+// kernel), while two warps' tables fit beside the largest unit (FP64 3c08 with a table of
+// 220 molecules' pairs 1.7 ms against 3.2 of the block kernel, one warp beside 230: 5.4
+// against 3.6).  32,000 molecules, 3c18 FP32 3.93 -> 1.01 ms a call; 15,001, 3c08 FP64
+// 3.74 -> 2.09; 7,811, 3c01 FP64 12.2 -> 3.9; vapours (8,000 molecules, densities 0.001
+// to 0.1) 0.2 to 0.9 of the others' times, but for 3c01 in FP64 with units of 14 to 32
+// molecules (1.03 to 1.25; of 61 0.84).
+// FP64: for r_c within 2^+-16, where the scan's FP32 products of six lengths are far
+// from the ends of their range (an r_c of 1e-9, in metres, would find no triplet); the
+// other kernels decide in FP64 what FP32 cannot.
 ProdLaunch atm_prod_plan(const ForceJob& j)
 {
     ProdLaunch l;
     if (j.trunc != 1 || j.trav < 0 || j.trav > 4 || j.trav == 3 || j.det || j.mcap < 1 || j.mcap > 65535 ||
-        (j.trav != 0 && j.mcap > ATM_MCAP_LIMIT) || (j.prec == 0 && (!j.x || j.rc_exp > PROD64_RC_EXP)))
+        (j.trav != 0 && j.mcap > ATM_MCAP_LIMIT) || (j.prec == 0 && (!j.x || j.rc_exp > PROD64_RC_EXP)) ||
+        (j.trav == 0 && j.prec == 0 && j.mcap < PROD64_OWNER_MIN))
         return l;
     const bool f64 = j.prec == 0;
     const long long fixed = f64 ? prod_smem<double>(j.trav, j.mcap).total : prod_smem<float>(j.trav, j.mcap).total;
@@ -252,11 +256,11 @@ ProdLaunch atm_prod_plan(const ForceJob& j)
     const long long lim = j.optin > 4096 ? (long long)j.optin - 4096 : 0;
     // an SM holds 20 (FP64) or 32 (FP32) warps of these kernels; four, three or two
     // CTAs to it while four warps' tables fit the largest unit and there are units
-    // for them
-    for (int c = f64 ? 2 : 4; c >= 1; c--) {
+    // for them; of units of up to 64 molecules, CTAs of four warps
+    for (int c = j.mcap <= 64 ? (f64 ? 5 : 8) : (f64 ? 2 : 4); c >= 1; c--) {
         const long long room = std::min<long long>(lim, 233472 / c - 2560);
         if (c > 1 && ((long long)j.b.ncell < (long long)c * j.sms || fixed + 4 * warp > room)) continue;
-        if (fixed + warp > room) return l;
+        if (fixed + 2 * warp > room) return l;
         l.warps = std::min<int>(PROD_MAXW, (f64 ? 20 : 32) / c);
         l.smem = (int)std::min<long long>(room, fixed + l.warps * warp);
         return l;
