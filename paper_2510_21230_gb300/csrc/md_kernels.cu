@@ -362,9 +362,8 @@ struct LjArith<float> {
 // molecules 327 -> 142, bound by the FP64 pipe.
 constexpr int LJ_PARTS = 8, LJ_TILE = 512;
 template <typename R>
-__global__ void __launch_bounds__(LJ_BLOCK) k_lj_owner(const LjArgs<R> A)
+__device__ __forceinline__ void lj_cell(const LjArgs<R>& A, const long long u)
 {
-    after_previous();
     typedef LjArith<R> Q;
     constexpr bool f64 = sizeof(R) == 8;
     constexpr unsigned FULL = 0xffffffffu;
@@ -373,7 +372,8 @@ __global__ void __launch_bounds__(LJ_BLOCK) k_lj_owner(const LjArgs<R> A)
     __shared__ int s_beg[28], s_g0[27];
     __shared__ float4 s_off[27];
     const int tid = threadIdx.x, lane = tid & 31;
-    const long long n = A.n, u = blockIdx.x;
+    const long long n = A.n;
+    if (A.cell_start[u] == A.cell_start[u + 1]) return;
     const Rep& rp = A.b.rep[A.b.rep_of_cell[u]];
     const int* st = A.cell_start + rp.cell0;
     int cx, cy, cz;
@@ -509,6 +509,29 @@ __global__ void __launch_bounds__(LJ_BLOCK) k_lj_owner(const LjArgs<R> A)
             A.mol_cnt[2 * s + 1] = pairs;
         }
     }
+}
+
+// One cell per CTA, or (MANY, in vapours) A.per of them, the empty ones passed over
+// together (20 molecules in a million cells: 870 us with a CTA each)
+template <typename R, bool MANY>
+__global__ void __launch_bounds__(LJ_BLOCK) k_lj_owner(const LjArgs<R> A)
+{
+    after_previous();
+    if constexpr (!MANY) {
+        lj_cell<R>(A, blockIdx.x);
+        return;
+    }
+    __shared__ unsigned s_full[LJ_BLOCK / 32];
+    const long long u0 = (long long)blockIdx.x * A.per, u = u0 + threadIdx.x;
+    const unsigned m = __ballot_sync(0xffffffffu, threadIdx.x < A.per && u < A.b.ncell &&
+                                                      A.cell_start[u] != A.cell_start[u + 1]);
+    if ((threadIdx.x & 31) == 0) s_full[threadIdx.x >> 5] = m;
+    __syncthreads();
+    for (int w = 0; w < LJ_BLOCK / 32; w++)
+        for (unsigned b = s_full[w]; b != 0u; b &= b - 1u) {
+            lj_cell<R>(A, u0 + 32 * w + __ffs(b) - 1);
+            __syncthreads();  // the tables are free
+        }
 }
 
 // ---------------------------------------------------------------- integrator
@@ -959,10 +982,17 @@ cudaError_t launch_lj(int prec, const LjArgs<double>& a64, const LjArgs<float>& 
 {
     long long n = prec == 0 ? a64.n : a32.n;
     if (n <= 0) return cudaSuccess;
+    const long long ncell = prec == 0 ? a64.b.ncell : a32.b.ncell;
+    LjArgs<double> l64 = a64;
+    LjArgs<float> l32 = a32;
+    l64.per = l32.per = (int)std::max(1ll, std::min<long long>(LJ_BLOCK, ncell / n));
+    const bool many = l64.per > 1;
     if (prec == 0)
-        launch_after(k_lj_owner<double>, (unsigned)a64.b.ncell, LJ_BLOCK, 0, st, a64);
+        launch_after(many ? k_lj_owner<double, true> : k_lj_owner<double, false>, nblk(ncell, l64.per), LJ_BLOCK, 0,
+                     st, l64);
     else
-        launch_after(k_lj_owner<float>, (unsigned)a32.b.ncell, LJ_BLOCK, 0, st, a32);
+        launch_after(many ? k_lj_owner<float, true> : k_lj_owner<float, false>, nblk(ncell, l32.per), LJ_BLOCK, 0, st,
+                     l32);
     return cudaGetLastError();
 }
 

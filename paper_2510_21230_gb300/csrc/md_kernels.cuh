@@ -14,6 +14,7 @@ struct LjArgs {
     double* fs;               // sorted-order LJ force, SoA [3n] (fully written)
     double* mol_ew;           // [2n] per sorted molecule: half of its pair energies, virials
     unsigned* mol_cnt;        // [2n] per sorted molecule: half-shell candidates, interacting pairs
+    int per = 1;              // cells of a CTA (set by the launch)
 };
 
 // device-side copy of atm_result (same layout)
