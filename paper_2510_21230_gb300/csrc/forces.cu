@@ -182,7 +182,7 @@ FwdLaunch atm_fwd_plan(const ForceJob& j)
     // LJ apart only for whole systems (in a domain the LJ kernel gives owned
     // molecules their complete force) and in floating point
     f.lj = j.lj && j.trav != 0 ? 1 : (j.lj_apart && j.whole && !j.det ? 2 : 0);
-    if (j.trav == 0 && f.lj != 2) return f;  // (no kernel of this form)
+    if (j.trav == 0 && f.lj != 2) return FwdLaunch();  // (no kernel of this form)
     // eight warps and a run of four cells per CTA; one cell, and several CTAs per
     // cell, while the grid would leave SMs without enough warps
     const long long sms = j.sms > 0 ? j.sms : 148, occ = (j.b.ntot + j.b.ncell - 1) / j.b.ncell;
@@ -205,7 +205,7 @@ FwdLaunch atm_fwd_plan(const ForceJob& j)
     }
     while (f.nwarps > 1 && !fits()) f.nwarps /= 2;
     f.use = fits();
-    return f;
+    return f.use ? f : FwdLaunch();  // (no LJ from lists that are not taken)
 }
 
 // The FP64 pair rule of 3c01, 3c18 and 3c08 on whole systems, outside the
@@ -228,7 +228,7 @@ FwdLaunch atm_list64_plan(const ForceJob& j)
     if (f.run == 1 && j.b.ncell < 4ll * j.sms && occ > FWD_MAXW) f.split = 2;
     if (list64_smem(j.mcap_fwd, f.run) > LIST64_SMEM) f.run = 1;
     f.use = list64_smem(j.mcap_fwd, f.run) <= LIST64_SMEM;
-    return f;
+    return f.use ? f : FwdLaunch();
 }
 
 // The product rule of 3c01, 3c18, 3c08 and 3c08a outside the deterministic mode (its
