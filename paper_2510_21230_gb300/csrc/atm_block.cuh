@@ -417,17 +417,14 @@ __device__ __forceinline__ void atm_block_unit(const AtmArgs<R>& A, const long l
         // broadcast load).  FP64: one warp per row, one ballot per 32 pairs
         // (the rare FP64 recomputations of the prefilter band stay spread
         // over the lanes).
-        if (!F64 && A.pmask) {
+        if (TRAV == 4 && !F64 && A.pmask) {
             // from the evaluation's pair bitmaps (k_pair_masks): word k - 13 of
             // a molecule covers the molecules of the cell at offset27(k), k =
             // 13 (its own cell, the later molecules) .. 26 (the forward
             // cells), in cell order, which is the staging order.  Slot s2
-            // lies at offset o(s2) - o(sp) from p's slot, and a later slot is
-            // a forward cell in both unit kinds (3c08: s = ox + 2 oy + 4 oz;
-            // 3c18: forward neighbours in lexicographic order), so row p of
-            // adj comes from p's own words.  Cells two apart (a 3c18 unit's
-            // outer slots) hold no pair within r_c: the host hands over
-            // bitmaps only when fl(w^2) >= the FP32 r_c^2 on every axis.
+            // lies at offset o(s2) - o(sp) from p's slot, and a later slot
+            // (s = ox + 2 oy + 4 oz) is a forward cell, so row p of adj comes
+            // from p's own words.
             for (int p = tid; p < M; p += blockDim.x) {
                 const int sp = sslot[p];
                 const long long gp = __float_as_int(P4[p].w);

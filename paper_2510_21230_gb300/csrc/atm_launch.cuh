@@ -25,9 +25,12 @@ AtmKernel<R> atm_kernel(int trav, int trunc)
         if (trav == 3 && trunc == 0) return atm_owner_kernel<3, 0, R>;
         if (trav == 3 && trunc == 1) return atm_owner_kernel<3, 1, R>;
     }
-    if (trav == 1 && trunc == 0) return atm_block_kernel<1, 0, R, DET>;
+    // (FP32, pair rule of 3c18 and 3c08: forward lists, which hold whatever these would)
+    if constexpr (sizeof(R) == 8) {
+        if (trav == 1 && trunc == 0) return atm_block_kernel<1, 0, R, DET>;
+        if (trav == 2 && trunc == 0) return atm_block_kernel<2, 0, R, DET>;
+    }
     if (trav == 1 && trunc == 1) return atm_block_kernel<1, 1, R, DET>;
-    if (trav == 2 && trunc == 0) return atm_block_kernel<2, 0, R, DET>;
     if (trav == 2 && trunc == 1) return atm_block_kernel<2, 1, R, DET>;
     if (trav == 4 && trunc == 0) return atm_block_kernel<4, 0, R, DET>;
     if (trav == 4 && trunc == 1) return atm_block_kernel<4, 1, R, DET>;

@@ -215,16 +215,6 @@ extern "C" atm_status atm_batch_create(const atm_params* params, const int64_t* 
     }
     c->n = ntot;
     c->ncell = ncell;
-    // a pair two cells apart is at least a cell edge w apart along that axis,
-    // and its FP32 squared distance at least fl(wf * wf): no pair within r_c
-    // when that is not below the FP32 r_c^2 (the 3c18 units' outer slots)
-    c->pm_3c18 = true;
-    for (const atm3::Rep& r : c->reps)
-        for (int d = 0; d < 3; d++) {
-            volatile float wf = r.wf[d];
-            volatile float w2 = wf * wf;
-            if (!(w2 >= r.rc2f)) c->pm_3c18 = false;
-        }
     auto alloc = [&](void** ptr, size_t bytes) -> bool {
         return cudaMalloc(ptr, bytes > 0 ? bytes : 16) == cudaSuccess;
     };
@@ -597,13 +587,11 @@ static void launch_choice(atm_ctx* c, int trav, int trunc, int prec, int mcap, i
         persistent = c->opt_persistent;
         nwarps = c->opt_nwarps;
         for (int k = 0; k < 3; k++) cls[k] = c->opt_cls[k];
-        if (nwarps == 0 && prec == ATM_FP32C && trunc == ATM_TRUNC_PAIR && !c->det &&
-            (trav == ATM_3C18 || trav == ATM_3C08 || trav == ATM_3C08A) && mcap > 0) {
+        if (nwarps == 0 && prec == ATM_FP32C && trunc == ATM_TRUNC_PAIR && !c->det && trav == ATM_3C08A && mcap > 0) {
             // without a tuned choice: 4 or 8 warps, whichever keeps more warps
-            // resident per SM for this unit size (4 on a tie).  Measured
-            // (256k / 32k liquids): 3c08 1.20 / 0.27 ms at 4 and 1.50 / 0.23 ms
-            // at 8 warps, 3c18 1.98 / 0.85 at 4 and 1.70 / 0.55 at 8.  (Not
-            // the deterministic mode: its 8-byte scalars change the balance,
+            // resident per SM for this unit size (4 on a tie; 256k / 32k liquids,
+            // units of 8 cells: 1.20 / 0.27 ms at 4 and 1.50 / 0.23 ms at 8 warps).
+            // (Not the deterministic mode: its 8-byte scalars change the balance,
             // and 8 warps measured slower there, 1.87 against 1.70 ms.)
             int* e = c->nw_auto[trav][trunc];
             const int band = mcap / 8 + 1;
@@ -637,12 +625,11 @@ static int edge_capacity(const atm_ctx* c, int trav, int trunc)
     return measured_edges(c, trav, trunc) ? c->gpm16[trav] : 256;
 }
 
-// FP32 pair rule of a block traversal, bitmaps enabled, every cell within 32
+// FP32 pair rule in the block kernel (3c08a), bitmaps enabled, every cell within 32
 static bool use_pair_masks(const atm_ctx* c, int trav, int trunc, int prec)
 {
     return c->opt_pmask && c->pmask && prec == ATM_FP32C && trunc == ATM_TRUNC_PAIR &&
-           (trav == ATM_3C08 || trav == ATM_3C08A || (trav == ATM_3C18 && c->pm_3c18)) &&
-           c->maxocc <= atm3::PM_CELL_MAX;
+           trav == ATM_3C08A && c->maxocc <= atm3::PM_CELL_MAX;
 }
 
 void atm3::ctx_want_list64(atm_ctx* c, int trav, int trunc, int prec, int mcap)

@@ -165,14 +165,14 @@ static cudaError_t launch_atm_one(const ForceJob& j, size_t* smem_set, bool* cap
 }
 
 // The FP32C pair rule of 3c01, 3c18 and 3c08 takes the forward lists (liquid of
-// 256,000 molecules at rho* 0.8, forces and LJ apart: 0.50 ms against 1.16 ms
-// of the pair bitmaps and the block kernel and 0.19 ms of the LJ kernel; five
-// steps 3.82 against 8.42 ms; 5,003 molecules 0.19 against 0.28 ms per call).
-// Left to the other kernels: 3c01 in parts of
-// a domain (owner computes: only owned molecules get a force) and in the
-// deterministic mode (its sums need no fixed point, so no term can leave the
-// fixed-point range), the corner-anchored 3c08 (not every triangle), and units
-// that do not fit shared memory.
+// 256,000 molecules at rho* 0.8: five steps 3.57 against 8.42 ms of the pair bitmaps
+// and the block kernel; 5,003 molecules 0.14 against 0.28 ms a call).  Left to the
+// owner kernel: 3c01 in parts of a domain (owner computes: only owned molecules get a
+// force) and in the deterministic mode (its sums need no fixed point, so no term can
+// leave the fixed-point range); to the block kernel: the corner-anchored 3c08 (not
+// every triangle).  Units that do not fit shared memory are refused before by the
+// block kernel's plan: 18 cells lie in four blocks of eight or two units of fourteen,
+// and its adjacency holds 900 molecules a unit, the lists 6,500.
 FwdLaunch atm_fwd_plan(const ForceJob& j)
 {
     FwdLaunch f;
@@ -330,8 +330,7 @@ static cudaError_t launch_fwd(const ForceJob& j, const FwdLaunch& f)
 
 bool atm_uses_pair_masks(const ForceJob& j)
 {
-    return j.pmask && !atm_fwd_plan(j).use && j.prec == 1 && j.trunc == 0 && (j.trav == 1 || j.trav == 2 || j.trav == 4) &&
-           j.b.ntot > 0;
+    return j.pmask && j.prec == 1 && j.trunc == 0 && j.trav == 4 && j.b.ntot > 0;
 }
 
 bool atm_split_active(const ForceJob& j)
