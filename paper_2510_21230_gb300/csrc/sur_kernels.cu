@@ -270,8 +270,7 @@ __global__ void __launch_bounds__(SUR_BLOCK, 5) k_sur_desc(const SurForceArgs A)
             const float r2 = dist2(row[j], sx, sy, sz, ex, ey, ez);
             word |= (r2 < kc.rc2 ? 1u : 0u) << (j & 31);
         }
-        const int self = t == 13 ? (int)s - q0 : -1;  // (the molecule itself)
-        if (self >= 0 && (!BIG || self < 32)) word &= ~(1u << (self & 31));
+        if (t == 13 && (!BIG || (int)s - q0 < 32)) word &= ~(1u << (((int)s - q0) & 31));  // (the molecule itself)
         mask[t * SUR_BLOCK + tid] = word;
         if constexpr (BIG) {
             word = 0u;
@@ -281,7 +280,7 @@ __global__ void __launch_bounds__(SUR_BLOCK, 5) k_sur_desc(const SurForceArgs A)
                 const float r2 = dist2(row[j], sx, sy, sz, ex, ey, ez);
                 word |= (r2 < kc.rc2 ? 1u : 0u) << (j - 32);
             }
-            if (self >= 32) word &= ~(1u << (self & 31));
+            if (t == 13 && (int)s - q0 >= 32) word &= ~(1u << (((int)s - q0) & 31));
             mask2[t * SUR_BLOCK + tid] = (unsigned short)word;
         }
         s_q0[t * SUR_BLOCK + tid] = q0;
@@ -292,22 +291,25 @@ __global__ void __launch_bounds__(SUR_BLOCK, 5) k_sur_desc(const SurForceArgs A)
         int t = -1, q0 = 0;
         unsigned bits = 0u, second = 0u;
         for (;;) {
-            while (bits == 0u) {
-                if (BIG && second != 0u) {
-                    bits = second;
-                    second = 0u;
-                    q0 += 32;
-                    break;
-                }
-                if (++t >= 27) break;
-                bits = mask[t * SUR_BLOCK + tid];
-                if constexpr (BIG) {
+            if constexpr (BIG) {
+                while (bits == 0u) {
+                    if (second != 0u) {
+                        bits = second;
+                        second = 0u;
+                        q0 += 32;
+                        break;
+                    }
+                    if (++t >= 27) break;
+                    bits = mask[t * SUR_BLOCK + tid];
                     second = mask2[t * SUR_BLOCK + tid];
                     q0 = s_q0[t * SUR_BLOCK + tid];
                 }
+                if (bits == 0u) break;
+            } else {
+                while (bits == 0u && ++t < 27) bits = mask[t * SUR_BLOCK + tid];
+                if (bits == 0u) break;
+                q0 = s_q0[t * SUR_BLOCK + tid];
             }
-            if (bits == 0u) break;
-            if constexpr (!BIG) q0 = s_q0[t * SUR_BLOCK + tid];
             const int q = q0 + __ffs(bits) - 1;
             bits &= bits - 1u;
             const float4 o = s_off[t];
