@@ -260,7 +260,8 @@ atm_status atm_get_results(atm_ctx* ctx, atm_result* out);
  * instead of one CTA per unit.  nwarps = 4 or 8 warps per 3C18/3C08 CTA (0 =
  * default); neither applies to the pair rule of 3C01, 3C18 and 3C08 (FP64:
  * outside the deterministic mode) and to the product rule outside the
- * deterministic mode (3CW apart), whose launch form follows from the system.
+ * deterministic mode (3CW and units beyond its kernel's tables apart), whose
+ * launch form follows from the system.
  * graph = 1: atm_step captures one step in a CUDA graph (on a
  * stream of its own) and replays it, with no host synchronisation between
  * steps; the graph sizes the kernels for the current largest unit plus
@@ -295,17 +296,19 @@ atm_status atm_set_owned_layers(atm_ctx* ctx, int replica, int z_lo, int z_hi);
  * virials vary at the rounding level from run to run: warps take work from
  * counters in the order they arrive and floating-point atomic additions
  * round in the order they happen).  In this mode
- *  - every warp takes its work in a fixed order (cell-triplet edge groups and
- *    candidate tasks of the block traversals, base molecules of 3C01 / 3CW),
- *    so each lane's energy and virial sums are the same every time;
- *  - the block traversals (3C18, 3C08, 3C08A) sum their pair scalars, their
- *    per-molecule fallback accumulators and the forces of different units as
- *    signed 64-bit integers in units of 2^-32 (FP32C) or 2^-44 (FP64): each
- *    term is rounded once to that grid and the sums do not depend on the
- *    order of the additions, so the forces are also the same for every launch
- *    form (one CTA per unit or persistent, warps per CTA, size classes);
- *    energies and virials then depend on the launch form only through the
- *    lanes' partial sums;
+ *  - every warp takes its work in a fixed order (the base cells' molecules of the
+ *    FP32C pair rule of 3C18 / 3C08, cell-triplet edge groups and candidate tasks
+ *    of the block kernel, base molecules of 3C01 / 3CW), so each lane's energy
+ *    and virial sums are the same every time;
+ *  - the block traversals (3C18, 3C08, 3C08A) sum as signed 64-bit integers in
+ *    units of 2^-32 (FP32C) or 2^-44 (FP64), each term rounded once to that
+ *    grid, so that the sums do not depend on the order of the additions.  FP32C
+ *    pair rule of 3C18 / 3C08: a term is what one molecule's triplets put on one
+ *    partner or on itself, an FP32 sum in a fixed order.  Otherwise: the pair
+ *    scalars, the per-molecule fallback accumulators and the forces of different
+ *    units.  The forces are thus the same for every launch form (one CTA per unit
+ *    or persistent, warps per CTA, size classes); energies and virials depend on
+ *    it only through the lanes' partial sums;
  *  - a term of size 2^26 (FP32C) or 2^14 = 16,384 (FP64) or more, which a
  *    liquid never reaches, makes the evaluation fail with ATM_E_RANGE.
  * 3C01 and 3CW write each force once (owner computes) and the LJ kernel owns
@@ -330,9 +333,13 @@ atm_status atm_set_deterministic(atm_ctx* ctx, int on);
 atm_status atm_set_pair_masks(atm_ctx* ctx, int on);
 
 /* Unit size classes of the block traversals (3C18, 3C08, 3C08A) for
- * evaluations and steps without an autotuned choice.  nclass = 1: every unit
- * in one launch sized for the largest unit (the default).  nclass = 2 or 3:
- * every force evaluation first lists, on the device, the units of at most
+ * evaluations and steps without an autotuned choice, where these run in the block
+ * kernel (the pair rule of 3C08A; FP64 pair rule of 3C18 and 3C08 in the
+ * deterministic mode, in parts of a domain and without lists; the product rule in
+ * the deterministic mode and for units beyond its kernel's tables): forward lists
+ * and the product kernel have no classes.
+ * nclass = 1: every unit in one launch sized for the largest unit (the default).
+ * nclass = 2 or 3: every force evaluation first lists, on the device, the units of at most
  * cuts[0] staged molecules, then (nclass = 3) those of at most cuts[1], then
  * the rest, and launches the block kernel once per class with shared memory
  * sized for the class bound (2 warps when it is at most 64): small units of
@@ -363,7 +370,7 @@ typedef struct {
  * sorts the units by their staged molecules on the device and launches each
  * class with shared memory sized for its bound, 2 warps for bounds up to 64)
  * and keeps the fastest for this (trav, trunc, prec); later evaluations and
- * steps use it.  Cells must be built.  out may be NULL.
+ * steps use it.  (One form is timed where atm_set_options' do not apply.)  Cells must be built.  out may be NULL.
  * Errors: INVALID, STATE, CAPACITY, CUDA. */
 atm_status atm_autotune(atm_ctx* ctx, atm_traversal trav, atm_truncation trunc,
                         atm_precision prec, int reps, atm_tuning* out);

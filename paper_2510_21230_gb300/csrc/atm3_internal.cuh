@@ -84,7 +84,8 @@ struct Batch {
 // Kernels of a step are launched with programmatic serialization (launch_after):
 // the next one's CTAs come to the SMs as the last of this one's leave them, and wait
 // here, before their first access to memory, for its end.  A call of 1,000
-// molecules is a chain of a dozen kernels of a few microseconds each: 143 -> 120 us a call.
+// molecules is a chain of a dozen kernels of a few microseconds each: 143 -> 120 us a call
+// (129 with the cell build's wait for its sort).
 __device__ __forceinline__ void after_previous()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -55,12 +55,12 @@
 // 256,000 molecules 3 % faster); the virial is 9 times the energy (u is homogeneous of
 // degree -9 in the distances).
 //
-// Bound by instruction issue (71 % of the issue slots on 32,000 molecules; 67 M
-// warp instructions there against 140 M of the block kernel).  256,000 molecules,
-// rho* = 0.8, lattice start, LJ apart: 0.50 ms against 1.35 ms of bitmaps, block
-// kernel and LJ kernel; of it, by leaving phases out, rounds 0.28, lists 0.07,
-// the rows' shares and LJ 0.10, staging and sums of the unit 0.04 (0.10 with one
-// base cell per CTA; lists of 33 in two chunks instead of 32 and 1: + 0.07).
+// Bound by instruction issue (72 % of the issue slots on 32,000 molecules, LJ apart:
+// 70 M warp instructions, 2.0 MB from DRAM, 0.090 ms; the block kernel 140 M).  256,000
+// molecules, rho* = 0.8, in a step (LJ inside): 0.47 ms against 1.16 ms of bitmaps and
+// block kernel; by leaving phases out, rounds are six tenths of it, lists 0.07 ms, the
+// rows' shares and LJ 0.10, staging and sums of the unit 0.04 (0.10 with one base cell
+// per CTA; lists of 33 in two chunks instead of 32 and 1: + 0.07).
 #pragma once
 #include <type_traits>
 

@@ -21,12 +21,12 @@
 // nearer row, it is 3 to 5.)  In a liquid 3c18 tests 24 % of its candidates.
 //   FP32  what is evaluated are the canonical displacements of the rows, as in the owner
 //         kernel (unit-frame positions are rounded at 2 w: rms force error up to a
-//         sixth more).  A lane evaluates its own hits, one a turn; nothing is queued, r's force
-//         stays in registers and p's too, q's goes to shared memory by three
-//         reductions.  A lane begins at its own bit of a word, and eight copies of
-//         the forces take the lanes in turn, for the far rows of a p share their
-//         few near ones (32,000 molecules, 3c18: 1.72 ms with one, 0.88 with four,
-//         0.86 with eight).  3c01 adds p's force compensated.
+//         sixth more).  A lane evaluates its own hits, one a turn; nothing is
+//         queued, r's force stays in registers and p's too (3c01: compensated),
+//         q's goes to shared memory by three reductions.  A lane begins at its own
+//         bit of a word, and eight copies of the forces take the lanes in turn,
+//         for the far rows of a p share their few near ones (32,000 molecules,
+//         3c18: 1.72 ms with one, 0.88 with four, 0.86 with eight).
 //   FP64  an instruction takes the FP64 pipe as long for one lane as for 32, so
 //         hits are queued, one a lane and turn, and evaluated 32 at a time; lanes
 //         hold the nearer row there (hits of one batch meet fewer equal rows).
@@ -39,9 +39,10 @@
 //
 // 32,000 molecules at density 0.8, 3c18, FP32: 0.86 ms (the block kernel: 3.69), issue
 // 55 % and the shared-memory reductions 50 % busy; with rows in staging order and hits
-// queued it took 2.1.  15,001 at 0.7, 3c08, FP64: 1.90 ms (3.36), bound by
-// the FP64 pipe, 69 instructions a triplet of which 43 are its arithmetic.  7,811, 3c01, FP64: 3.8 ms
-// a call (12.2).
+// queued it took 2.1.  15,001 at 0.7, 3c08, FP64: 1.86 ms (3.36), bound by the FP64
+// pipe, 69 instructions a triplet of which 43 are its arithmetic.  7,811, 3c01, FP64:
+// 3.8 ms a call (12.2).  Units of up to 64 molecules run in CTAs of four warps (see
+// atm_prod_plan).
 //
 // Decisions.  Squares from unit-frame positions are within 2.4e-4 (relative) of
 // the canonical FP32 and FP64 ones for sides above 0.02 w, and c = a + b - 2 q.r
@@ -124,6 +125,7 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
     __shared__ int s_beg[S + 1];
     __shared__ int s_cell0[S];
     __shared__ signed char s_off[S][3];
+    __shared__ float4 s_offf[F64 ? 1 : S];
     __shared__ int s_next, s_dmin, s_rows;
     __shared__ double s_red[2][PROD_MAXW];
     __shared__ unsigned long long s_redn[PROD_MAXW];
@@ -178,6 +180,7 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
     for (int s = warp; s < S; s += nwarps) {
         const int b = s_beg[s], e = s_beg[s + 1], g0 = s_cell0[s] - b;
         const int ox = s_off[s][0], oy = s_off[s][1], oz = s_off[s][2];
+        if (!F64 && lane == 0) s_offf[s] = make_float4((float)ox, (float)oy, (float)oz, 0.0f);
         // images of the cells beyond the box edges
         const double sx = cx + ox < 0 ? -rp.g.L[0] : (cx + ox >= rp.g.nc[0] ? rp.g.L[0] : 0.0);
         const double sy = cy + oy < 0 ? -rp.g.L[1] : (cy + oy >= rp.g.nc[1] ? rp.g.L[1] : 0.0);
@@ -352,14 +355,17 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
             py = X[M + p];
             pz = X[2 * M + p];
         }
-        // FP32: the rows that are evaluated are the canonical displacements
+        // FP32: the rows that are evaluated are the canonical displacements (3c08, 256,000
+        // molecules: 8.2 ms, 7.7 from unit-frame positions; cell-local positions in shared
+        // memory instead of read again: 3c08 at 32,000 1.37 ms for 1.46, 3c18 0.97 for 0.91)
         float lx = 0.0f, ly = 0.0f, lz = 0.0f;
-        const int sp = __float_as_int(P.w);
+        float4 op = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if constexpr (!F64) {
             const long long g = sidx[p];
             lx = A.xl[g];
             ly = A.xl[n + g];
             lz = A.xl[2 * n + g];
+            op = s_offf[__float_as_int(P.w)];
         }
         const int first = OWNER ? 0 : p + 1;
         bins[lane] = 0;
@@ -391,13 +397,12 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
                 to[4] = V.z;
                 to[6] = b;
                 if constexpr (!F64) {
-                    const long long g = sidx[t];
-                    const int s = __float_as_int(S4[t].w);
-                    float dx, dy, dz;
-                    canon_disp<float>(lx, ly, lz, A.xl[g], A.xl[n + g], A.xl[2 * n + g], s_off[s][0] - s_off[sp][0],
-                                      s_off[s][1] - s_off[sp][1], s_off[s][2] - s_off[sp][2], rp.wf[0], rp.wf[1],
-                                      rp.wf[2], dx, dy, dz);
-                    rows4[k] = make_float4(dx, dy, dz, __int_as_float(t));
+                    const float* xg = A.xl + sidx[t];
+                    const float4 o = s_offf[__float_as_int(V.w)];
+                    rows4[k] = make_float4(__fadd_rn(__fsub_rn(xg[0], lx), __fmul_rn(o.x - op.x, rp.wf[0])),
+                                           __fadd_rn(__fsub_rn(xg[n], ly), __fmul_rn(o.y - op.y, rp.wf[1])),
+                                           __fadd_rn(__fsub_rn(xg[2 * n], lz), __fmul_rn(o.z - op.z, rp.wf[2])),
+                                           __int_as_float(t));
                 } else {
                     rid[k] = (unsigned short)t;
                 }
