@@ -92,9 +92,10 @@ typedef enum { ATM_TRUNC_PAIR = 0, ATM_TRUNC_PRODUCT = 1 } atm_truncation;
  *         triplets, each evaluated once at its lowest molecule i on the canonical
  *         displacements from i; what the triplets of i put on one partner is a
  *         plain FP32 sum (3C01: compensated), and the shares of different i are
- *         added in FP64.  The product rule of 3C01, 3C18, 3C08 and 3C08A takes the
- *         canonical displacements from a triplet's first molecule; a unit's forces
- *         are plain FP32 sums, those of different units are added in FP64 (3C01:
+ *         added in FP64.  The product rule of 3C01 and 3C18 takes the canonical
+ *         displacements from a triplet's first molecule, that of 3C08 and 3C08A
+ *         the FP32-rounded unit-frame positions xl + o w; a unit's forces are
+ *         plain FP32 sums, those of different units are added in FP64 (3C01:
  *         compensated (Kahan) FP32 per-lane sums of F_i, combined in FP64).  The
  *         pair rule of 3C08A takes the FP32-rounded unit-frame positions xl + o w and
  *         adds each triplet's three pair scalars to per-edge FP32 sums, then each

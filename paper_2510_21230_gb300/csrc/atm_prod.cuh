@@ -19,9 +19,11 @@
 // that hold the farther row have hits alike: the longest list of 32 lanes is 1.5
 // to 1.8 of their mean; with rows in staging order, or lanes that hold the
 // nearer row, it is 3 to 5.)  In a liquid 3c18 tests 24 % of its candidates.
-//   FP32  what is evaluated are the canonical displacements of the rows, as in the owner
-//         kernel (unit-frame positions are rounded at 2 w: rms force error up to a
-//         sixth more).  A lane evaluates its own hits, one a turn; nothing is
+//   FP32  3c01 and 3c18 evaluate the canonical displacements of the rows, as the owner
+//         kernel does (unit-frame positions, rounded at 2 w, gave 3c01 up to 9 % more
+//         rms force error and 3c18 up to 4 than the kernels before; 3c08 and 3c08a
+//         are below those with them, and 7 % faster than with canonical rows).  A
+//         lane evaluates its own hits, one a turn; nothing is
 //         queued, r's force stays in registers and p's too (3c01: compensated),
 //         q's goes to shared memory by three reductions.  A lane begins at its own
 //         bit of a word, and eight copies of the forces take the lanes in turn,
@@ -119,14 +121,15 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
 {
     constexpr int S = Trav<TRAV>::S;
     constexpr bool F64 = sizeof(R) == 8, OWNER = TRAV == 0;
+    constexpr bool CANON = !F64 && (TRAV == 0 || TRAV == 1);  // evaluates canonical displacements
     constexpr bool TABLE = F64 && (TRAV == 2 || TRAV == 4);  // dense pair scalars
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_beg[S + 1];
     __shared__ int s_cell0[S];
     __shared__ signed char s_off[S][3];
-    __shared__ float4 s_offf[F64 ? 1 : S];
-    __shared__ int s_next, s_dmin, s_rows;
+    __shared__ float4 s_offf[CANON ? S : 1];
+    __shared__ int s_next, s_dmin, s_rows, s_none;
     __shared__ double s_red[2][PROD_MAXW];
     __shared__ unsigned long long s_redn[PROD_MAXW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -145,10 +148,14 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
         return;
     }
     if (warp == 0) unit_slots<TRAV, S>(rp.g, A.cell_start + rp.cell0, lu, s_beg, s_cell0, s_off);
-    if (tid == 0) {
-        s_next = 0;
-        s_dmin = 0x7f000000;
-        s_rows = 0;
+    if (warp == 0) {
+        __syncwarp();
+        if (lane == 0) {
+            s_next = 0;
+            s_dmin = 0x7f000000;
+            s_rows = 0;
+            s_none = s_beg[S] < 3;
+        }
     }
     __syncthreads();
     const int M = s_beg[S];
@@ -158,13 +165,10 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
         store_zero();
         return;
     }
-    if (Mp == 0 || M < 3) {  // no triplet, and no candidate but of other corners' anchored sets
-        if (warp == 0) {
-            const unsigned long long cand =
-                OWNER ? (lane == 0 ? unit_candidates<TRAV, S>(s_beg) : 0ull) : unit_candidates_warp<TRAV, S>(s_beg);
-            store_zero();
-            if (tid == 0) A.unit_cnt[2 * u] = cand;
-        }
+    // no triplet, and no candidate (all of them hold a p); 3c08 is told by shared memory (the
+    // test on M itself costs its FP32 kernel registers and 4 % of its time, and saves 3c18 2 %)
+    if (TRAV == 2 ? s_none : M < 3 || Mp == 0) {
+        store_zero();
         return;
     }
     const ProdSmem plan = prod_smem<R>(TRAV, M);
@@ -180,7 +184,7 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
     for (int s = warp; s < S; s += nwarps) {
         const int b = s_beg[s], e = s_beg[s + 1], g0 = s_cell0[s] - b;
         const int ox = s_off[s][0], oy = s_off[s][1], oz = s_off[s][2];
-        if (!F64 && lane == 0) s_offf[s] = make_float4((float)ox, (float)oy, (float)oz, 0.0f);
+        if (CANON && lane == 0) s_offf[s] = make_float4((float)ox, (float)oy, (float)oz, 0.0f);
         // images of the cells beyond the box edges
         const double sx = cx + ox < 0 ? -rp.g.L[0] : (cx + ox >= rp.g.nc[0] ? rp.g.L[0] : 0.0);
         const double sy = cy + oy < 0 ? -rp.g.L[1] : (cy + oy >= rp.g.nc[1] ? rp.g.L[1] : 0.0);
@@ -355,17 +359,12 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
             py = X[M + p];
             pz = X[2 * M + p];
         }
-        // FP32: the rows that are evaluated are the canonical displacements (3c08, 256,000
-        // molecules: 8.2 ms, 7.7 from unit-frame positions; cell-local positions in shared
-        // memory instead of read again: 3c08 at 32,000 1.37 ms for 1.46, 3c18 0.97 for 0.91)
-        float lx = 0.0f, ly = 0.0f, lz = 0.0f;
-        float4 op = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if constexpr (!F64) {
-            const long long g = sidx[p];
-            lx = A.xl[g];
-            ly = A.xl[n + g];
-            lz = A.xl[2 * n + g];
-            op = s_offf[__float_as_int(P.w)];
+        float lx = 0.0f, ly = 0.0f, lz = 0.0f;  // CANON: p lies in the base cell
+        if constexpr (CANON) {
+            const float* xp = A.xl + sidx[p];
+            lx = xp[0];
+            ly = xp[n];
+            lz = xp[2 * n];
         }
         const int first = OWNER ? 0 : p + 1;
         bins[lane] = 0;
@@ -396,13 +395,15 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
                 to[2] = V.y;
                 to[4] = V.z;
                 to[6] = b;
-                if constexpr (!F64) {
+                if constexpr (CANON) {
                     const float* xg = A.xl + sidx[t];
                     const float4 o = s_offf[__float_as_int(V.w)];
-                    rows4[k] = make_float4(__fadd_rn(__fsub_rn(xg[0], lx), __fmul_rn(o.x - op.x, rp.wf[0])),
-                                           __fadd_rn(__fsub_rn(xg[n], ly), __fmul_rn(o.y - op.y, rp.wf[1])),
-                                           __fadd_rn(__fsub_rn(xg[2 * n], lz), __fmul_rn(o.z - op.z, rp.wf[2])),
+                    rows4[k] = make_float4(__fadd_rn(__fsub_rn(xg[0], lx), __fmul_rn(o.x, rp.wf[0])),
+                                           __fadd_rn(__fsub_rn(xg[n], ly), __fmul_rn(o.y, rp.wf[1])),
+                                           __fadd_rn(__fsub_rn(xg[2 * n], lz), __fmul_rn(o.z, rp.wf[2])),
                                            __int_as_float(t));
+                } else if constexpr (!F64) {
+                    rows4[k] = make_float4(V.x, V.y, V.z, __int_as_float(t));
                 } else {
                     rid[k] = (unsigned short)t;
                 }
@@ -444,7 +445,7 @@ __device__ __forceinline__ void atm_prod_unit(const AtmArgs<R>& A, const long lo
             float Vx = 0.0f, Vy = 0.0f, Vz = 0.0f, b = 0.0f;
             int ri = p, v = 0;
             if (own) {
-                if constexpr (F64) {
+                if constexpr (!CANON) {
                     const float* vr = rows + 8 * (r >> 1) + (r & 1);
                     Vx = vr[0];
                     Vy = vr[2];
