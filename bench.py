@@ -95,25 +95,21 @@ F2_FUSED = 27.0
 FUSED_TRAV = ("3c08", "3c18", "3c08a")
 
 # DRAM traffic per ATM evaluation (dram__bytes_read.sum + dram__bytes_write.sum
-# of its kernels -- the FP32C pair rule's pair-bitmap kernel and the block
-# kernel -- from one ncu capture, whose replays start from a flushed L2: the
-# bitmaps the block kernel reads count as DRAM bytes there, though a run finds
-# them in L2), keyed by (traversal, truncation, precision, workload), with the
-# sha256 prefix of the kernel sources it was taken from: a changed kernel
-# reports null until it is captured again.  liquid_n256k is the N = 32,000
-# capture (2197 units) scaled to 19683 units.
+# of its kernel in a step, LJ inside, from one ncu capture on the lattice start,
+# whose replays start from a flushed L2), keyed by (traversal, truncation,
+# precision, workload), with the sha256 prefix of the kernel sources it was
+# taken from: a changed kernel reports null until it is captured again.
 KERNEL_SOURCES = ["atm3_internal.cuh", "atm_common.cuh", "atm_block.cuh", "atm_owner.cuh",
                   "atm_fp32.cu", "atm_fp64.cu", "atm_launch.cuh", "pair_masks.cu", "atm_fwd.cuh",
                   "atm_fwd.cu", "atm_list64.cu", "atm_prod.cuh", "atm_prod.cu"]
-TRAFFIC = {("3c08", "pair", "fp32c", "liquid_n256k"): (32.43e6, "86ebe58ae46bedf4"),
-           ("3c08", "pair", "fp32c", "liquid_n32k"): (3.620e6, "86ebe58ae46bedf4")}
+TRAFFIC = {("3c08", "pair", "fp32c", "liquid_n256k"): (9.839e6, "482d62eede82c86b")}
 
 
 # Issued FP32 flops (fadd + fmul + 2 ffma thread instructions of the ATM
-# evaluation's kernels, from the same ncu capture) over its useful flops,
-# with the source hash they belong to: what candidates and bookkeeping add
-# in floating point.
-ISSUED = {("3c08", "pair", "fp32c"): (0.929, "86ebe58ae46bedf4")}
+# evaluation's kernel, from the same ncu capture) over its useful flops,
+# with the source hash they belong to: what candidates, masked pairs of the
+# lists and bookkeeping add in floating point.
+ISSUED = {("3c08", "pair", "fp32c"): (2.383, "482d62eede82c86b")}
 
 
 def kernel_hash():
