@@ -485,13 +485,13 @@ static void take_unit_sizes(atm_ctx* c)
     }
 }
 
-// cell build + read back of the occupancy maxima that size the force kernels
-static atm_status enqueue_cells(atm_ctx* c)
+// cell build + read back of the occupancy maxima that size the force kernels; the
+// host waits for the sizes, or (idle) for the sort behind them too
+static atm_status enqueue_cells(atm_ctx* c, bool idle = false)
 {
-    // the host waits for the sizes, not for the sort behind them
     atm_status s = launch_cells(c, true);
     if (s != ATM_OK) return s;
-    CU(cudaEventSynchronize(c->ev_occ));
+    CU(idle ? cudaStreamSynchronize(c->st) : cudaEventSynchronize(c->ev_occ));
     if (c->ev_live.size() >= 4096) prof_drain(c);
     s = check_status(c);
     if (s != ATM_OK) return s;
@@ -516,12 +516,9 @@ extern "C" atm_status atm_build_cells(atm_ctx* c)
     if (!c) return ATM_E_INVALID;
     if (!c->have_x) return ctx_fail(c, ATM_E_STATE, "no state set");
     CU(cudaSetDevice(c->device));
-    const atm_status s = enqueue_cells(c);
-    if (s != ATM_OK) return s;
     // (a step goes on while the molecules are sorted; this call returns with the
     // stream idle)
-    CU(cudaStreamSynchronize(c->st));
-    return ATM_OK;
+    return enqueue_cells(c, true);
 }
 
 extern "C" atm_status atm_get_cells(atm_ctx* c, int32_t* cell_of, int32_t* cell_start,
